@@ -156,6 +156,7 @@ void free_axis(AxisData& a) {
   dfree(a.tw);
   dfree(a.tw32);
   for (void* q : a.bs) dfree(q);
+  dfree(a.mtw);
   for (float* q : a.gemm) dfree(q);
   a = AxisData{};
 }
@@ -312,14 +313,14 @@ int build_axis_aux(helm_plan* p, AxisData& a, double rho, int q) {
 
 // Bluestein tables of an axis whose length has a prime factor above 64, in
 // the compute precision `prec`: the chirp w_j = e^{i pi j^2/n} (j^2 reduced
-// mod 2n in integers), the length-m DFTs of the chirp sequence b (b_j = w_j
-// for |j| < n, cyclic) for the forward transform and of conj(b) for the
-// inverse one, both divided by m, and the length-m twiddles.  FP64 on the
-// host (the spectra by a direct O(m^2) sum).
+// mod 2n in integers), the length-m DFT of the chirp sequence b (b_j = w_j
+// for |j| < n, cyclic) divided by m, and the length-m twiddles.  FP64 on the
+// host (the spectrum by a direct O(m^2) sum).
 int build_bluestein(helm_plan* p, AxisData& a, int prec) {
-  const int64_t n = a.n, m = bluestein_length(n);
+  const int64_t n = a.n, m = mix_bluestein(n, bluestein_length(n), prec, &a.dft.mix);
+  if (!m) return HELM_EUNSUPPORTED;
   const double pi = 3.14159265358979323846;
-  std::vector<std::complex<double>> w(n), b(m, 0.0), f0(m), f1(m);
+  std::vector<std::complex<double>> w(n), b(m, 0.0), f0(m);
   for (int64_t j = 0; j < n; ++j) {
     const int64_t r = (j * j) % (2 * n);
     w[j] = std::polar(1.0, pi * (double)r / (double)n);
@@ -329,15 +330,12 @@ int build_bluestein(helm_plan* p, AxisData& a, int prec) {
   std::vector<double> rre(m), rim(m);
   unit_roots(m, rre.data(), rim.data());  // e^{-2 pi i k/m}
   for (int64_t k = 0; k < m; ++k) {
-    std::complex<double> s0 = 0.0, s1 = 0.0;
+    std::complex<double> s0 = 0.0;
     for (int64_t j = 0; j < m; ++j) {
       const int64_t e = (j * k) % m;
-      const std::complex<double> t(rre[e], rim[e]);
-      s0 += b[j] * t;
-      s1 += std::conj(b[j]) * t;
+      s0 += b[j] * std::complex<double>(rre[e], rim[e]);
     }
     f0[k] = s0 / (double)m;
-    f1[k] = s1 / (double)m;
   }
   const size_t es = prec == kPrecF64 ? sizeof(double2) : sizeof(float2);
   auto put = [&](void** dst, const std::vector<std::complex<double>>& v) -> int {
@@ -351,18 +349,13 @@ int build_bluestein(helm_plan* p, AxisData& a, int prec) {
   };
   std::vector<std::complex<double>> twm(m);
   for (int64_t k = 0; k < m; ++k) twm[k] = {rre[k], rim[k]};
+  w.resize(m, 0.0);  // the points past a line's end are read times zero
   int rc;
-  if ((rc = put(&a.bs[0], w)) || (rc = put(&a.bs[1], f0)) || (rc = put(&a.bs[2], f1)) || (rc = put(&a.bs[3], twm)))
-    return rc;
-  DftPlan mp;
-  dft_factor(m, &mp);
+  if ((rc = put(&a.bs[0], w)) || (rc = put(&a.bs[1], f0)) || (rc = put(&a.bs[2], twm))) return rc;
   a.dft.bm = (int)m;
-  a.dft.bstages = mp.nstages;
-  for (int s = 0; s < mp.nstages; ++s) a.dft.bradix[s] = mp.radix[s];
   a.dft.bw = a.bs[0];
-  a.dft.bf[0] = a.bs[1];
-  a.dft.bf[1] = a.bs[2];
-  a.dft.btw = a.bs[3];
+  a.dft.bf = a.bs[1];
+  a.dft.btw = a.bs[2];
   return HELM_OK;
 }
 
@@ -374,8 +367,20 @@ int build_axis(helm_plan* p, AxisData& a, int64_t n, double h, double wc, double
   a.h = h;
   a.wc = wc;
   dft_factor(n, &a.dft);
-  if (dft_needs_bluestein(a.dft))
-    if (int rc = build_bluestein(p, a, p->prec)) return rc;
+  if (!dft_needs_bluestein(a.dft)) mix_plan(n, p->prec, &a.dft.mix);
+  else if (int rc = build_bluestein(p, a, p->prec)) return rc;
+  if (p->prec == kPrecF32) {
+    std::vector<std::complex<double>> t;
+    mix_tables(a.dft.mix, &t);
+    std::vector<float> t32;
+    for (const std::complex<double>& z : t) {
+      t32.push_back((float)z.real());
+      t32.push_back((float)z.imag());
+    }
+    if (t32.empty()) t32.resize(2);  // a single pass has no twiddles
+    if (int rc = upload32(p, &a.mtw, t32)) return rc;
+    a.dft.mtw = a.mtw;
+  }
   std::vector<double> twre(n), twim(n);
   unit_roots(n, twre.data(), twim.data());
   std::vector<double> tw(2 * n), lamA(2 * n), sigA(2 * n), parA(n);
@@ -1888,6 +1893,7 @@ int helm_solve_2d_static(int64_t nx, int64_t ny, double hx, double hy, double om
   ax.h = hy;
   ax.wc = omega;
   dft_factor(ny, &ax.dft);
+  mix_plan(ny, kPrecF64, &ax.dft.mix);
   int dev = 0, smem = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kStaticMaxDevices ||
       cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {

@@ -19,7 +19,8 @@ enum { kInC64 = 0, kInC128 = 1, kInFF = 2 };
 
 bool dft_supported(const DftPlan& p, size_t elem_bytes, int max_smem);
 // A length whose factorisation has a prime above 64 is transformed by
-// Bluestein's chirp-z method; its power-of-two convolution length (>= 2n - 1).
+// Bluestein's chirp-z method; the largest convolution length it may take (the
+// power of two >= 2n - 1).
 bool dft_needs_bluestein(const DftPlan& p);
 
 // Tensor-core (tcgen05, kind::tf32 with high/low operand splitting) dense
@@ -69,6 +70,17 @@ bool dft_cols_pow2_supported(int64_t n);
 cudaError_t launch_dft_cols_pow2(int prec, const void* in, int in_is_double, void* out, int out_mode, int64_t outer,
                                  int64_t inner, int64_t n, const void* tw, int sign, double scale, double accum_scale,
                                  const void* sc_in, const void* sc_out, const int* skip, cudaStream_t st);
+
+// Lines of any supported length by the mixed-radix passes p.mix: the
+// contracts of launch_dft_rows and launch_dft_cols (in place allowed; complex64
+// columns read complex64).
+cudaError_t launch_dft_rows_mix(int prec, const void* in, int in_is_double, void* out, int out_mode, int64_t nrows,
+                                const DftPlan& p, const void* tw, int sign, double scale, double accum_scale,
+                                const void* sc_in, const void* sc_out, const int* skip, cudaStream_t st);
+cudaError_t launch_dft_cols_mix(int prec, const void* in, int in_is_double, void* out, int out_mode, int64_t outer,
+                                int64_t inner, const DftPlan& p, const void* tw, int sign, double scale,
+                                double accum_scale, const void* sc_in, const void* sc_out, const int* skip,
+                                cudaStream_t st);
 
 // Lines along a middle axis: the array viewed as [outer][p.n][inner].
 cudaError_t launch_dft_cols(int prec, const void* in, int in_is_double, void* out, int out_mode,

@@ -15,6 +15,7 @@
 
 #include "helm_async.cuh"
 #include "helm_dft.h"
+#include "helm_dft_radix.cuh"
 #include "helm_kernels.cuh"
 
 namespace helm {
@@ -26,105 +27,6 @@ __device__ __forceinline__ C twid(const C* __restrict__ tw, int e) {
   C w = __ldg(&tw[e]);  // forward table e^{-2 pi i e / n}
   if (SIGN > 0) w.y = -w.y;
   return w;
-}
-
-// (SIGN i) a
-template <typename C, int SIGN>
-__device__ __forceinline__ C mul_si(C a) {
-  C o;
-  if (SIGN > 0) {
-    o.x = -a.y;
-    o.y = a.x;
-  } else {
-    o.x = a.y;
-    o.y = -a.x;
-  }
-  return o;
-}
-
-// (cr + i ci) a for compile-time constants
-template <typename C>
-__device__ __forceinline__ C mul_c(C a, double cr, double ci) {
-  using T = decltype(a.x);
-  C o;
-  o.x = a.x * (T)cr - a.y * (T)ci;
-  o.y = a.x * (T)ci + a.y * (T)cr;
-  return o;
-}
-
-// In-register R-point DFTs, natural order in and out:
-// y_q = sum_r v_r e^{SIGN 2 pi i r q / R}.
-template <typename C, int SIGN>
-__device__ __forceinline__ void dft2(C* v) {
-  const C a = v[0];
-  v[0] = cadd(a, v[1]);
-  v[1] = csub(a, v[1]);
-}
-
-template <typename C, int SIGN>
-__device__ __forceinline__ void dft4s(C& v0, C& v1, C& v2, C& v3) {
-  const C t0 = cadd(v0, v2), t1 = csub(v0, v2), t2 = cadd(v1, v3), t3 = mul_si<C, SIGN>(csub(v1, v3));
-  v0 = cadd(t0, t2);
-  v1 = cadd(t1, t3);
-  v2 = csub(t0, t2);
-  v3 = csub(t1, t3);
-}
-
-template <typename C, int SIGN>
-__device__ __forceinline__ void dft4(C* v) {
-  dft4s<C, SIGN>(v[0], v[1], v[2], v[3]);
-}
-
-constexpr double kH = 0.70710678118654752440;   // cos(pi/4)
-constexpr double kC8 = 0.92387953251128675613;  // cos(pi/8)
-constexpr double kS8 = 0.38268343236508977173;  // sin(pi/8)
-
-template <typename C, int SIGN>
-__device__ __forceinline__ void dft8(C* v) {
-  // even and odd halves: E_q in v[2q], O_q in v[2q+1]
-  dft4s<C, SIGN>(v[0], v[2], v[4], v[6]);
-  dft4s<C, SIGN>(v[1], v[3], v[5], v[7]);
-  const double s = SIGN;
-  const C o1 = mul_c(v[3], kH, s * kH);     // W8^1 O_1
-  const C o2 = mul_si<C, SIGN>(v[5]);       // W8^2 O_2
-  const C o3 = mul_c(v[7], -kH, s * kH);    // W8^3 O_3
-  const C e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6], o0 = v[1];
-  v[0] = cadd(e0, o0);
-  v[4] = csub(e0, o0);
-  v[1] = cadd(e1, o1);
-  v[5] = csub(e1, o1);
-  v[2] = cadd(e2, o2);
-  v[6] = csub(e2, o2);
-  v[3] = cadd(e3, o3);
-  v[7] = csub(e3, o3);
-}
-
-template <typename C, int SIGN>
-__device__ __forceinline__ void dft16(C* v) {
-  // r = b + 4a: DFT4 over a for each b (results Z_b[q1] at v[b + 4 q1])
-#pragma unroll
-  for (int b = 0; b < 4; ++b) dft4s<C, SIGN>(v[b], v[b + 4], v[b + 8], v[b + 12]);
-  // twiddles W16^{b q1}
-  const double s = SIGN;
-  v[5] = mul_c(v[5], kC8, s * kS8);     // b1 q1 = 1
-  v[9] = mul_c(v[9], kH, s * kH);       // b1 q2 = 2
-  v[13] = mul_c(v[13], kS8, s * kC8);   // b1 q3 = 3
-  v[6] = mul_c(v[6], kH, s * kH);       // b2 q1 = 2
-  v[10] = mul_si<C, SIGN>(v[10]);       // b2 q2 = 4
-  v[14] = mul_c(v[14], -kH, s * kH);    // b2 q3 = 6
-  v[7] = mul_c(v[7], kS8, s * kC8);     // b3 q1 = 3
-  v[11] = mul_c(v[11], -kH, s * kH);    // b3 q2 = 6
-  v[15] = mul_c(v[15], -kC8, -s * kS8); // b3 q3 = 9
-  // DFT4 over b for each q1: y[q1 + 4 q2] lands at v[4 q1 + q2]
-#pragma unroll
-  for (int q1 = 0; q1 < 4; ++q1) dft4s<C, SIGN>(v[4 * q1], v[4 * q1 + 1], v[4 * q1 + 2], v[4 * q1 + 3]);
-  C y[16];
-#pragma unroll
-  for (int q1 = 0; q1 < 4; ++q1)
-#pragma unroll
-    for (int q2 = 0; q2 < 4; ++q2) y[q1 + 4 * q2] = v[4 * q1 + q2];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = y[i];
 }
 
 template <typename C, int R, int SIGN>

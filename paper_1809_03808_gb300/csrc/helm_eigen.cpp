@@ -369,9 +369,8 @@ int dft_factor(int64_t n, DftPlan* p) {
   p->n = (int)n;
   p->nstages = 0;
   p->bm = 0;
-  p->bstages = 0;
-  p->bw = p->btw = nullptr;
-  p->bf[0] = p->bf[1] = nullptr;
+  p->bw = p->bf = p->btw = p->mtw = nullptr;
+  p->mix = MixPlan{};
   p->gw[0] = p->gw[1] = nullptr;
   p->gsc[0] = p->gsc[1] = nullptr;
   p->gscale = 0.0;

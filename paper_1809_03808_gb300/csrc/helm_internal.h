@@ -1,8 +1,10 @@
 // Internal declarations shared by the host plan code and the CUDA kernels.
 #pragma once
 
+#include <complex>
 #include <cstddef>
 #include <cstdint>
+#include <vector>
 
 #include <cuda_runtime.h>
 
@@ -22,23 +24,38 @@ void dfree(void* ptr);
 // (a plan build beside a served solve) cannot lower it under one another.
 cudaError_t allow_dynamic_smem(const void* func, size_t bytes);
 
+// One pass of a mixed-radix transform of n points: radix r, nb = n / r
+// butterflies, span ns (the product of the earlier radices), twiddle stride
+// st = n / (ns r), where its twiddles (toff) and a prime's roots (roff) begin
+// in the complex64 tables, and the multipliers of the divisions by nb and ns.
+struct MixStage {
+  int r, nb, ns, st, toff, roff;
+  uint32_t mnb, mns;
+};
+constexpr int kMixStages = 9;
+struct MixPlan {
+  int n, nstages;
+  int mid;  // Bluestein: the pass that ends the first transform and begins the second (-1: none)
+  MixStage s[kMixStages];
+};
+
 // Mixed-radix factorisation of a DFT length: 8, 4, 2 first, then odd primes.
 struct DftPlan {
   int n;
   int nstages;
   int radix[kMaxStages];
-  // Lengths with a prime factor above 64 (Bluestein's chirp-z transform):
-  // bm = the power-of-two convolution length (0: not used), its radices, and
-  // device tables in the plan's compute precision: bw the chirp
-  // e^{i pi j^2 / n} (n values), bf[0] / bf[1] the length-bm DFT of the chirp
-  // sequence for the forward / inverse transform, scaled by 1/bm, btw the
-  // twiddles e^{-2 pi i k / bm}.
+  // Passes of the mixed-radix kernels (helm_dft_mix.cu), of length n or, for
+  // lengths with a prime factor above 64 (Bluestein's chirp-z transform), of
+  // the convolution length bm >= 2n - 1 (0: not used) there and back.  Its
+  // device tables in the plan's compute precision: bw the chirp e^{i pi j^2 / n}
+  // (n values, then zeros up to bm), bf the length-bm DFT of the chirp sequence divided by bm, btw
+  // the twiddles e^{-2 pi i k / bm} (complex128).
+  MixPlan mix;
   int bm;
-  int bstages;
-  int bradix[kMaxStages];
   const void* bw;
-  const void* bf[2];
+  const void* bf;
   const void* btw;
+  const void* mtw;  // complex64: mix_tables of mix
   // Tensor-core variant (complex64 lines of at most 128 points): gw[0] /
   // gw[1] the forward / inverse matrix tables of launch_dft_rows_tc (null:
   // not built), made with the FP32 scalings gsc[0] (input, forward) and
@@ -50,6 +67,16 @@ struct DftPlan {
 };
 
 int dft_factor(int64_t n, DftPlan* p);
+
+// The passes of a transform of n points (nstages = 0: a prime factor above
+// 64), and of Bluestein's transform of n points on the cheapest convolution
+// length in [2n - 1, top], which is returned.
+// prec: kPrecF64 or kPrecF32.
+void mix_plan(int64_t n, int prec, MixPlan* m);
+int64_t mix_bluestein(int64_t n, int64_t top, int prec, MixPlan* m);
+// The passes' twiddle tables: per pass s > 0 [ns][r] values e^{-2 pi i k q /
+// (ns r)}, then the r roots e^{-2 pi i q / r} of a pass of a prime above 10.
+void mix_tables(const MixPlan& m, std::vector<std::complex<double>>* out);
 
 // Eigen-data of the absorbing 1D pencil (see helm_eigen.cpp).
 // mden: the mass matrix denominator (6: the paper's elements, 12: the
@@ -96,7 +123,8 @@ struct AxisData {
   double* parA = nullptr;   // +-1 : V[n,l] = par * V[1,l]
   double* tw = nullptr;     // e^{-2 pi i k/n} (re, im) interleaved, FP64
   float* tw32 = nullptr;    // same, FP32
-  void* bs[4] = {nullptr, nullptr, nullptr, nullptr};  // Bluestein tables of dft (chirp, 2 spectra, twiddles)
+  void* bs[3] = {nullptr, nullptr, nullptr};  // Bluestein tables of dft (chirp, spectrum, twiddles)
+  float* mtw = nullptr;                       // mix_tables of dft.mix (complex64 plans)
   float* gemm[2] = {nullptr, nullptr};                  // tensor-core DFT tables of dft (forward, inverse)
   DftPlan dft{};
 };
