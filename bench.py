@@ -205,9 +205,9 @@ def kernel_model(name, e, n1, accum=False, first=True, tables=False, ff=False, p
         # refined paths: the first solve writes u (16 B), the sweeps update it (32 B)
         "dft_inv": (e + ((16.0 + (per_solve - 1.0) * 32.0) / per_solve if accum else 16 if e == 16 else 8),
                     5.0 * log2n),
-        # f, u complex128 in, r complex64 out; FP64 instructions per unknown of
-        # the monomial form (2D: 3 sums, 4 multiply-adds, ... = 14; 3D: 26)
-        "residual_fp64": (40.0, 14.0 if n1_dim == 2 else 26.0),
+        # f, u complex128 in, r complex64 out; 64-bit fixed point on the integer
+        # pipes: no FP64 instructions in its loop
+        "residual_fp64": (40.0, 0.0),
         # f, u float-float (16 B each) in, r complex64 out
         "residual_ff": (40.0, 40.0),
         "split_ff": (40.0, 4.0),  # f in, float-float f and its hi parts out
@@ -226,11 +226,11 @@ NCU_TRAFFIC_PER_UNKNOWN = {
         (546.5e6 + 118.0e6 + 2.5e6) / (4096 * 4096),
         "ncu --set full, 4096 x 4096: k_residual2d_ff + k_perimeter2d_ff "
         "(profiles/ncu_2d_kernels_4096x4096.md)"),
-    # DRAM bytes of one k_residual3d_tma launch on 256^3 (same spacing and wave
-    # number), per unknown; the traffic of a launch is proportional to them
+    # DRAM bytes of one k_residual3d_fx launch on 128 x 512 x 512, per unknown;
+    # the traffic of a launch is proportional to them
     ("3d", "c64_refined", "residual_fp64"): (
-        (569.948416e6 + 118.337536e6) / 256 ** 3,
-        "ncu --set full, 256^3: k_residual3d_tma (profiles/ncu_residual3d_tma_256cube.md), scaled by unknowns"),
+        (1107.046656e6 + 252.338432e6) / (128 * 512 * 512),
+        "ncu, 128 x 512 x 512: k_residual3d_fx (profiles/ncu_residual3d_fx.md), scaled by unknowns"),
 }
 
 
@@ -249,7 +249,7 @@ def roofline_entry(name, launches, tot_ms, steps, N, e, n1, peaks, fp64, accum=F
     hbm_frac = gbs / hbm if hbm else None
     # the binding resource: FP64 arithmetic for FP64 kernels unless the HBM
     # fraction is the larger one
-    if (fp64 or name == "residual_fp64") and (hbm_frac is None or alu_frac >= hbm_frac):
+    if fp64 and (hbm_frac is None or alu_frac >= hbm_frac):
         out.update({"bound": "alu", "achieved": tfl, "peak": FP64_PEAK_TFLOPS, "unit": "T FP64-op/s",
                     "frac": alu_frac, "peak_source": FP64_PEAK_NOTE,
                     "algorithmic_flops_per_launch": flops, "algorithmic_bytes_per_launch": byts,

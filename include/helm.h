@@ -58,7 +58,9 @@ enum helm_dtype {
 };
 
 /* Arithmetic of the refinement residual r = f - A u (HELM_C64_REFINED).
- *   HELM_RESID_FP64  u accumulated in complex128, residual in FP64.
+ *   HELM_RESID_FP64  u accumulated in complex128, residual of the complex128
+ *                    vectors in 64-bit fixed point with a scale per tile: its
+ *                    rounding is below FP64's own of the tile's largest terms.
  *   HELM_RESID_FF    f and u held as float-float pairs (hi + lo floats, about
  *                    48 significant bits), residual and accumulation on the
  *                    FP32 pipes; u converted to complex128 once at the end.

@@ -13,6 +13,7 @@
 
 #include "helm_async.cuh"
 #include "helm_kernels.cuh"
+#include "helm_resid.h"
 #include "helm_solve.h"
 
 namespace helm {
@@ -46,10 +47,11 @@ struct ResidFFArgs {
 };
 
 // ---------------------------------------------------------------------------
-// FP64 residual with the fewest FP64 instructions.  On this GPU an FP64
-// instruction costs the SM about as much issue time as 64 FP32 ones, so the
-// stencil is rearranged to minimise them; everything else (staging, norms,
-// conversions) runs on the FP32 and integer pipes.
+// The stencil as sums of neighbours, and its FP64 form with the fewest FP64
+// instructions (an FP64 instruction costs the SM about as much issue time as
+// 64 FP32 ones).  Solves take the fixed-point kernels of helm_resid_fx.cu,
+// which use the same coefficients (512^3: 2.4 ms against 8.1); k_residual3d_q
+// remains for 3D arrays that no tensor map can describe.
 //
 // Per axis k the 1D matrices of eqs. matrixK / matrixM are
 //   M_k = m0 I + m1 S_k,  K_k = k0 I + k1 S_k,
@@ -85,17 +87,6 @@ __device__ __forceinline__ float round_d2f(double x) {
   const bool up = rem > 0x10000000u || (rem == 0x10000000u && (top & 1u));
   return __uint_as_float((sgn | ((uint32_t)(e - 896) << 23) | top) + (up ? 1u : 0u));
 }
-
-struct ResidQArgs {
-  int64_t n[3];
-  // 3D: c0[4 cx + 2 cy + cz][2 b + c], c1[2 cy + cz][2 b + c]; 2D: c0[2 cx + cy][b], c1[cy][b]
-  double2 c0[8][4];
-  double2 c1[4][4];
-  // 3D corrections of the end classes against the same class inside y and z:
-  // dc0[cls][bc] = c0[cls][bc] - c0[cls & 4][bc], dc1[cyz][bc] = c1[cyz][bc] - c1[0][bc]
-  double2 dc0[8][4];
-  double2 dc1[4][4];
-};
 
 // (acc.x, acc.y) += c v
 __device__ __forceinline__ void cadd_mul(double2& acc, double2 c, double2 v) {
@@ -243,137 +234,6 @@ __global__ void __launch_bounds__(QZ* QY) k_residual3d_q(ResidQArgs a, const dou
   block_norms<QZ * QY>(r2f, f2f, sums, ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x);
 }
 
-// The same 3D residual with the u planes brought in by the tensor memory
-// accelerator: one thread issues a tiled load of the plane's (QY+2) x (QZ+2)
-// halo box, whose parts outside the grid arrive as zeros, so the staging
-// needs no per-thread index or bounds arithmetic and no registers.  Three
-// plane buffers: while plane i is used, planes i+1 and i+2 are in flight; the
-// z sums are double-buffered, so one barrier per plane separates every reuse.
-// The plane's f tile comes by the same kind of load on the same barrier.
-// Every wait is bounded: a copy that does not arrive sets *err, the whole CTA
-// stops, and thread 0 lets its copies still in flight land before it exits.
-constexpr int QUB = (QY + 2) * (QZ + 2) * (int)sizeof(double2);  // bytes of one staged u plane
-constexpr int QUS = (QUB + 127) / 128 * 128;                      // its stride (TMA destinations: 128 B)
-constexpr int QFB = QY * QZ * (int)sizeof(double2);               // bytes of one f plane tile
-constexpr int QNB = 3;                                            // plane buffers
-constexpr int QSZB = 2 * (QY + 2) * QZ * (int)sizeof(double2);    // the two z-sum buffers
-constexpr size_t kResidTmaSmem = (size_t)QNB * (QUS + QFB) + QSZB + QNB * sizeof(uint64_t);
-
-__global__ void __launch_bounds__(QZ* QY, 2)
-    k_residual3d_tma(const __grid_constant__ CUtensorMap umap, const __grid_constant__ CUtensorMap fmap, ResidQArgs a,
-                     float2* __restrict__ r, double* __restrict__ sums, const int* __restrict__ skip, int* err) {
-  if (skip && *skip) return;
-  extern __shared__ __align__(128) unsigned char rsm[];
-  unsigned char* sUb = rsm;                                               // [QNB][QUS] u halo planes
-  unsigned char* sFb = sUb + QNB * QUS;                                   // [QNB][QFB] f plane tiles
-  double2(*sSz)[QY + 2][QZ] = reinterpret_cast<double2(*)[QY + 2][QZ]>(sFb + QNB * QFB);  // [2]
-  uint64_t* bar = reinterpret_cast<uint64_t*>(sFb + QNB * QFB + QSZB);
-  const int64_t nx = a.n[0], ny = a.n[1], nz = a.n[2];
-  const int tz = threadIdx.x, ty = threadIdx.y, tid = ty * QZ + tz;
-  const int64_t z0 = (int64_t)blockIdx.x * QZ, y0 = (int64_t)blockIdx.y * QY;
-  const int64_t xs = (int64_t)blockIdx.z * QX, xe = min(xs + QX, nx);
-  const int np = (int)(xe - xs + 2);  // planes xs-1 .. xe (at least 3)
-  const int64_t gz = z0 + tz, gy = y0 + ty;
-  const bool own = gz < nz && gy < ny;
-  const int cy = (gy == 0 || gy == ny - 1) ? 1 : 0, cz = (gz == 0 || gz == nz - 1) ? 1 : 0;
-  const int cyz = 2 * cy + cz;
-  const double2 zero = make_double2(0.0, 0.0);
-  float r2f = 0.f, f2f = 0.f;
-  if (tid == 0) {
-    for (int b = 0; b < QNB; ++b) mbar_init(&bar[b], 1);
-    fence_mbar_init();
-  }
-  __syncthreads();
-  // plane xs - 1 + i of u (halo box) and of f (the tile) into buffer i % QNB
-  // (thread 0 only; boxes outside the grid arrive as zeros)
-  auto issue = [&](int i) {
-    const int b = i % QNB;
-    mbar_arrive_expect_tx(&bar[b], (uint32_t)(QUB + QFB));
-    tma_load_3d(sUb + b * QUS, &umap, (int)(2 * (z0 - 1)), (int)(y0 - 1), (int)(xs - 1 + i), &bar[b]);
-    tma_load_3d(sFb + b * QFB, &fmap, (int)(2 * z0), (int)y0, (int)(xs - 1 + i), &bar[b]);
-  };
-  int issued = 0;
-  if (tid == 0) {
-    issue(0);
-    issue(1);
-    issued = 2;
-  }
-  double2 Rm = zero, Rc = zero, Qc = zero;  // R(x-2), R(x-1), f - Q at x-1
-  int i = 0;
-  bool failed = false;
-  for (; i < np; ++i) {
-    const int64_t ip = xs - 1 + i;
-    const double2* U = reinterpret_cast<const double2*>(sUb + (i % QNB) * QUS);  // [QY+2][QZ+2]
-    const double2* F = reinterpret_cast<const double2*>(sFb + (i % QNB) * QFB);  // [QY][QZ]
-    double2(*Sz)[QZ] = sSz[i & 1];
-    const bool outp = own && ip >= xs && ip < xe;
-    const bool got = mbar_wait_bounded(&bar[i % QNB], (uint32_t)((i / QNB) & 1), err);
-    for (int e = tid; e < (QY + 2) * QZ; e += QZ * QY) {
-      const int yy = e / QZ, zc = e - yy * QZ;
-      const double2 lo = U[yy * (QZ + 2) + zc], hi = U[yy * (QZ + 2) + zc + 2];
-      Sz[yy][zc] = make_double2(lo.x + hi.x, lo.y + hi.y);
-    }
-    if (__syncthreads_or(!got)) {  // block-uniform
-      failed = true;
-      break;
-    }
-    // every thread is past plane i - 1: its buffers take plane i + 2
-    if (tid == 0 && i + 2 < np) {
-      issue(i + 2);
-      issued = i + 3;
-    }
-    const double2 fv = outp ? F[ty * QZ + tz] : zero;
-    double2 Rn = zero, Qn = fv;
-    if (own && ip >= 0 && ip < nx) {
-      const double2 P00 = U[(ty + 1) * (QZ + 2) + tz + 1], P01 = Sz[ty + 1][tz];
-      const double2 ym = U[ty * (QZ + 2) + tz + 1], yp = U[(ty + 2) * (QZ + 2) + tz + 1];
-      const double2 sm = Sz[ty][tz], sp = Sz[ty + 2][tz];
-      const double2 P10 = make_double2(ym.x + yp.x, ym.y + yp.y), P11 = make_double2(sm.x + sp.x, sm.y + sp.y);
-      const int cx = (ip == 0 || ip == nx - 1) ? 1 : 0;
-      Rn.x = fma(a.c1[0][3].x, P11.x, fma(a.c1[0][2].x, P10.x, fma(a.c1[0][1].x, P01.x, a.c1[0][0].x * P00.x)));
-      Rn.y = fma(a.c1[0][3].x, P11.y, fma(a.c1[0][2].x, P10.y, fma(a.c1[0][1].x, P01.y, a.c1[0][0].x * P00.y)));
-      if (outp) {
-        if (cx == 0) {
-          Qn.x = fma(-a.c0[0][3].x, P11.x, fma(-a.c0[0][2].x, P10.x, fma(-a.c0[0][1].x, P01.x, fma(-a.c0[0][0].x, P00.x, Qn.x))));
-          Qn.y = fma(-a.c0[0][3].x, P11.y, fma(-a.c0[0][2].x, P10.y, fma(-a.c0[0][1].x, P01.y, fma(-a.c0[0][0].x, P00.y, Qn.y))));
-        } else {
-          csub_mul(Qn, a.c0[4][0], P00);
-          csub_mul(Qn, a.c0[4][1], P01);
-          csub_mul(Qn, a.c0[4][2], P10);
-          csub_mul(Qn, a.c0[4][3], P11);
-        }
-      }
-      if (cyz) {
-        if (cy | cz) cadd_mul(Rn, a.dc1[cyz][0], P00);
-        if (cy) cadd_mul(Rn, a.dc1[cyz][1], P01);
-        if (cz) cadd_mul(Rn, a.dc1[cyz][2], P10);
-        if (outp) {
-          const int cls = 4 * cx + cyz;
-          if (cy | cz) csub_mul(Qn, a.dc0[cls][0], P00);
-          if (cy) csub_mul(Qn, a.dc0[cls][1], P01);
-          if (cz) csub_mul(Qn, a.dc0[cls][2], P10);
-        }
-      }
-    }
-    const int64_t ix = ip - 1;
-    if (own && ix >= xs && ix < xe) {
-      const float2 rf = make_float2(round_d2f(Qc.x - Rm.x - Rn.x), round_d2f(Qc.y - Rm.y - Rn.y));
-      r[(ix * ny + gy) * nz + gz] = rf;
-      r2f = fmaf(rf.x, rf.x, fmaf(rf.y, rf.y, r2f));
-    }
-    if (outp) {
-      const float fx = round_d2f(fv.x), fy = round_d2f(fv.y);
-      f2f = fmaf(fx, fx, fmaf(fy, fy, f2f));
-    }
-    Rm = Rc;
-    Rc = Rn;
-    Qc = Qn;
-  }
-  if (failed && tid == 0)
-    for (int j = i; j < issued; ++j) mbar_wait_bounded(&bar[j % QNB], (uint32_t)((j / QNB) & 1), nullptr);
-  block_norms<QZ * QY>(r2f, f2f, sums, ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x);
-}
-
 // The driver's tensor-map encoder, looked up once through the runtime (no
 // link-time dependence on the driver library); null if unavailable.
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
@@ -390,9 +250,8 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   return fn;
 }
 
-// Tensor map of a [nx][ny][nz] complex128 array viewed as [nx][ny][2 nz]
-// FP64, with a box of bz complex values x by rows along y; false if it cannot
-// be made (the caller then stages the planes with plain loads).
+}  // namespace
+
 bool residual_map(CUtensorMap* m, const double2* v, const int64_t* n, int bz, int by) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
   if (!enc || ((uintptr_t)v & 15) || 2 * n[2] > (int64_t)UINT32_MAX || n[1] > (int64_t)UINT32_MAX ||
@@ -407,78 +266,7 @@ bool residual_map(CUtensorMap* m, const double2* v, const int64_t* n, int bz, in
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// 2D: thread per y column, QR2 rows rolling along x; monomials P_0 = u,
-// P_1 = Sy u of each row; r(x) = f(x) - Q(x) - R(x-1) - R(x+1).
-constexpr int QR2 = 32;
-__global__ void __launch_bounds__(256) k_residual2d_q(ResidQArgs a, const double2* __restrict__ f,
-                                                      const double2* __restrict__ u, float2* __restrict__ r,
-                                                      double* __restrict__ sums, const int* __restrict__ skip) {
-  if (skip && *skip) return;
-  const int64_t nx = a.n[0], ny = a.n[1];
-  const int64_t iy = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t xs = (int64_t)blockIdx.y * QR2, xe = min(xs + QR2, nx);
-  const bool own = iy < ny;
-  const int cy = (iy == 0 || iy == ny - 1) ? 1 : 0;
-  const double2 zero = make_double2(0.0, 0.0);
-  float r2f = 0.f, f2f = 0.f;
-  double2 Rm = zero, Rc = zero, Qc = zero;
-  if (own) {
-    const bool ym = iy > 0, yp = iy < ny - 1;
-    // row loads one row ahead
-    double2 c0v = zero, cmv = zero, cpv = zero, fv = zero;
-    auto load = [&](int64_t ix, double2& c, double2& m, double2& p) {
-      c = m = p = zero;
-      if (ix >= 0 && ix < nx) {
-        const double2* row = u + ix * ny + iy;
-        c = __ldg(row);
-        if (ym) m = __ldg(row - 1);
-        if (yp) p = __ldg(row + 1);
-      }
-    };
-    load(xs - 1, c0v, cmv, cpv);
-    for (int64_t ip = xs - 1; ip <= xe; ++ip) {
-      const double2 P0 = c0v;
-      const double2 P1 = make_double2(cmv.x + cpv.x, cmv.y + cpv.y);
-      const bool outp = ip >= xs && ip < xe;
-      if (outp) fv = __ldg(&f[ip * ny + iy]);
-      if (ip + 1 <= xe) load(ip + 1, c0v, cmv, cpv);
-      double2 Rn = zero, Qn = fv;
-      if (ip >= 0 && ip < nx) {
-        const int cx = (ip == 0 || ip == nx - 1) ? 1 : 0;
-        if (cy == 0 && cx == 0) {
-          Rn.x = fma(a.c1[0][1].x, P1.x, a.c1[0][0].x * P0.x);
-          Rn.y = fma(a.c1[0][1].x, P1.y, a.c1[0][0].x * P0.y);
-          if (outp) {
-            Qn.x = fma(-a.c0[0][1].x, P1.x, fma(-a.c0[0][0].x, P0.x, Qn.x));
-            Qn.y = fma(-a.c0[0][1].x, P1.y, fma(-a.c0[0][0].x, P0.y, Qn.y));
-          }
-        } else {
-          csub_mul(Rn, a.c1[cy][0], P0);
-          csub_mul(Rn, a.c1[cy][1], P1);
-          Rn = make_double2(-Rn.x, -Rn.y);
-          if (outp) {
-            csub_mul(Qn, a.c0[2 * cx + cy][0], P0);
-            csub_mul(Qn, a.c0[2 * cx + cy][1], P1);
-          }
-        }
-      }
-      const int64_t ix = ip - 1;
-      if (ix >= xs && ix < xe) {
-        const float2 rf = make_float2(round_d2f(Qc.x - Rm.x - Rn.x), round_d2f(Qc.y - Rm.y - Rn.y));
-        r[ix * ny + iy] = rf;
-        r2f = fmaf(rf.x, rf.x, fmaf(rf.y, rf.y, r2f));
-      }
-      if (outp) {
-        const float fx = round_d2f(fv.x), fy = round_d2f(fv.y);
-        f2f = fmaf(fx, fx, fmaf(fy, fy, f2f));
-      }
-      Rm = Rc;
-      Rc = Rn;
-      Qc = Qn;
-    }
-  }
-  block_norms<256>(r2f, f2f, sums, (int64_t)blockIdx.y * gridDim.x + blockIdx.x);
-}
+namespace {
 
 // ---------------------------------------------------------------------------
 // Float-float residual r = f - A u (f and u as float-float complex vectors,
@@ -907,9 +695,8 @@ cudaError_t launch_residual(int dim, const int64_t* n, const double* h, double o
                             const double2* f,
                             const double2* u, float2* r, double* sums, int64_t* nblocks, const int* skip,
                             cudaStream_t st, int* err, double mden) {
-  const int bs = 256;
   if (dim == 2 || dim == 3) {
-    // monomial coefficients by end class (see the FP64-instruction-lean kernels)
+    // monomial coefficients by end class
     ResidQArgs q{};
     for (int k = 0; k < dim; ++k) q.n[k] = n[k];
     using cd = std::complex<double>;
@@ -940,14 +727,11 @@ cudaError_t launch_residual(int dim, const int64_t* n, const double* h, double o
           if (cls < 4)
             q.dc1[cls][bc] = make_double2(q.c1[cls][bc].x - q.c1[0][bc].x, q.c1[cls][bc].y - q.c1[0][bc].y);
         }
+      const cudaError_t e = launch_residual_fx(3, q, f, u, r, sums, nblocks, skip, err, st);
+      if (e != cudaErrorNotSupported) return e;
       const dim3 grid((unsigned)((n[2] + QZ - 1) / QZ), (unsigned)((n[1] + QY - 1) / QY), (unsigned)((n[0] + QX - 1) / QX));
       *nblocks = (int64_t)grid.x * grid.y * grid.z;
-      CUtensorMap um, fm;
-      const cudaError_t attr = allow_dynamic_smem((const void*)k_residual3d_tma, kResidTmaSmem);
-      if (attr == cudaSuccess && residual_map(&um, u, n, QZ + 2, QY + 2) && residual_map(&fm, f, n, QZ, QY))
-        k_residual3d_tma<<<grid, dim3(QZ, QY), kResidTmaSmem, st>>>(um, fm, q, r, sums, skip, err);
-      else
-        k_residual3d_q<<<grid, dim3(QZ, QY), 0, st>>>(q, f, u, r, sums, skip);
+      k_residual3d_q<<<grid, dim3(QZ, QY), 0, st>>>(q, f, u, r, sums, skip);
       return cudaGetLastError();
     }
     for (int cx = 0; cx < 2; ++cx)
@@ -958,10 +742,7 @@ cudaError_t launch_residual(int dim, const int64_t* n, const double* h, double o
             if (a1 == 0) put(q.c0[2 * cx + cy][b], v);
             else if (cx == 0) put(q.c1[cy][b], v);
           }
-    const dim3 grid((unsigned)((n[1] + bs - 1) / bs), (unsigned)((n[0] + QR2 - 1) / QR2));
-    *nblocks = (int64_t)grid.x * grid.y;
-    k_residual2d_q<<<grid, bs, 0, st>>>(q, f, u, r, sums, skip);
-    return cudaGetLastError();
+    return launch_residual_fx(2, q, f, u, r, sums, nblocks, skip, err, st);
   }
   return cudaErrorInvalidValue;
 }
@@ -1113,14 +894,13 @@ cudaError_t launch_refine_init(RefineState* st, double tol, int max_iter, cudaSt
 
 int64_t residual_blocks(int dim, const int64_t* n) {
   if (dim == 2) {
-    // the larger of the FP64 grid and the float-float interior + perimeter grids
-    const int64_t fp64 = ((n[1] + 255) / 256) * ((n[0] + QR2 - 1) / QR2);
+    // the larger of the fixed-point grid and the float-float interior + perimeter grids
     const int64_t ff = ((n[1] - 2 + 255) / 256) * ((n[0] - 2 + RX2 - 1) / RX2) + (2 * n[1] + 2 * (n[0] - 2) + 255) / 256;
-    return std::max(fp64, ff);
+    return std::max(residual_fx_blocks(2, n), ff);
   }
   const int64_t ff = ((n[2] + TZ3 - 1) / TZ3) * ((n[1] + TY3 - 1) / TY3) * ((n[0] + RX3 - 1) / RX3);
   const int64_t q = ((n[2] + QZ - 1) / QZ) * ((n[1] + QY - 1) / QY) * ((n[0] + QX - 1) / QX);
-  return std::max(ff, q);
+  return std::max(std::max(ff, q), residual_fx_blocks(3, n));
 }
 
 cudaError_t launch_residual_finalize(const double* sums, int64_t nblocks, RefineState* state,

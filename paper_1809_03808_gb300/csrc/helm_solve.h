@@ -84,7 +84,8 @@ struct RefineState {
   double resid[16];
 };
 
-// r = f - A u in FP64 (eq. A2D / A3D), r stored as complex64, per-block sums
+// r = f - A u of FP64 vectors (eq. A2D / A3D) in 64-bit fixed point, at least
+// FP64's accuracy (helm_resid_fx.cu), r stored as complex64, per-block sums
 // of |r|^2 and |f|^2 into `sums` (2 doubles per block).  Returns the number of
 // blocks used through *nblocks.
 // wc[k]: w of the absorbing ends of axis k (0 on a Neumann axis).  err: the
