@@ -43,9 +43,7 @@ struct Plane3DArgs {
 
 constexpr int XC = 32;  // rows per reduction chunk
 
-constexpr int kMW = 16;       // inner modes per tile
-constexpr int kLineVals = 5;  // per-line table values (see k_plane_tables)
-constexpr int kPivRows = 32;  // pivot rows staged in shared memory (rows below a line's settling row)
+constexpr int kLineVals = 6;  // per-line table values (see k_plane_tables)
 constexpr int kRoutedFlag = 1 << 30;  // in the settling-row table: the line is solved in FP64
 // Routing is off by default: the complex64 solve's error does sit in the
 // near-singular lines (92 % of it in 1 % of the lines on a 160^3 grid of the
@@ -448,9 +446,9 @@ __global__ void k_outer_cbb(const typename cpx<T>::type* __restrict__ v, const t
 // complex128), so the tiled sweeps read the table only for rows < len and use
 // 1/u_inf beyond.  Per line (kLineVals values, line = l * nz + m): 1/u_inf,
 // 1/u_{nx-1} (the corner row), the off-diagonal b of the line matrix, and
-// the carry coefficients alpha, beta of a chunk of ch settled rows (see
-// k_inner3d), all from the FP64 values.  For propagating modes the
-// pivots keep oscillating and len covers the whole line.
+// the carry coefficients alpha, beta of a chunk of ch settled rows and beta of
+// the line's last chunk (see k_inner3d), all from the FP64 values.  For
+// propagating modes the pivots keep oscillating and len covers the whole line.
 
 template <typename T>
 __global__ void k_plane_tables(typename cpx<T>::type* __restrict__ tab, typename cpx<T>::type* __restrict__ lend,
@@ -474,12 +472,19 @@ __global__ void k_plane_tables(typename cpx<T>::type* __restrict__ tab, typename
   double2 c = make_double2(0, 0);
   int64_t last_bad = -1;
   double2 inv = make_double2(0, 0);
+  const int64_t slast = (nx - 1) / ch * ch;  // first row of the last chunk
+  double2 all = make_double2(1, 0), bel = make_double2(0, 0);
   for (int64_t ix = 0; ix < nx; ++ix) {
     const double2 aj = (ix == 0 || ix == nx - 1) ? k.ac : k.a;
     const double2 den = ix == 0 ? aj : csub(aj, cmul(k.b, c));
     inv = crecip(den);
     c = cmul(k.b, inv);
     tab[ix * ny * nz + i] = cvt<C>(inv);
+    if (ix >= slast) {  // g_j = -b / u_j
+      const double2 an = cmul(all, make_double2(-c.x, -c.y));
+      bel = cadd(bel, cmul(all, an));
+      all = an;
+    }
     if (ix < nx - 1) {
       const double dx = inv.x - iinf.x, dy = inv.y - iinf.y;
       if (!(dx * dx + dy * dy <= tol2)) last_bad = ix;
@@ -500,6 +505,7 @@ __global__ void k_plane_tables(typename cpx<T>::type* __restrict__ tab, typename
     lend[kLineVals * i + 2] = cvt<C>(k.b);
     lend[kLineVals * i + 3] = cvt<C>(al);
     lend[kLineVals * i + 4] = cvt<C>(be);
+    lend[kLineVals * i + 5] = cvt<C>(bel);
     lenL[i] = (int)(last_bad + 1);
   }
 }
@@ -552,26 +558,41 @@ Plane3DArgs make_args(const Plan3D& p) {
 // (the lines (x, l, m0..m0+kMW-1), x = 0..nx-1).  It stages their right-hand
 // sides in shared memory ([x][kMW], read from HBM once), and solves each line
 // by the chunked LU of Section 4.1.2's per-mode solves: thread (m, c) owns rows
-// [c*ch, c*ch + ch) of line m.
-//   pass 1: with the carries d_{s-1} = 0, x_{e+1} = 0 the chunk's forward
-//     substitution d_j = (r_j - b d_{j-1}) / u_j gives d_loc at its last row
-//     and, through the running products alpha_j = prod_{i<=j} (-b / u_i), the
-//     backward substitution's value x_loc at its first row, plus the
-//     rhs-independent alpha_e and beta = sum_j alpha_{j-1} alpha_j, so that
-//       d_e = d_loc + alpha_e d_{s-1},
-//       x_s = x_loc + beta d_{s-1} + alpha_e x_{e+1};
+// [c*ch, c*ch + ch) of line m.  With g_j = -b / u_j and running products
+// p_j = prod_{i<j} g_i over the chunk:
+//   pass 1 (carries d_{s-1} = 0 and x_{e+1} = 0): the forward substitution
+//     d_j = r_j / u_j + g_j d_{j-1} ends in d_loc, the backward one
+//     x_j = d_j + g_j x_{j+1} in x_loc at the chunk's first row; with
+//     alpha = p_{e+1} and beta = sum_j p_j p_{j+1},
+//       d_e = d_loc + alpha d_{s-1},
+//       x_s = x_loc + beta d_{s-1} + alpha x_{e+1};
 //   scan: these affine maps composed over the chunks of each line by one warp
 //     (Kogge-Stone over lanes), forward for d and backward for x;
-//   pass 2: the chunk's substitutions again from the exact carries; d and then
-//     x overwrite the staged right-hand sides.
+//   pass 2: d_j += p_{j+1} d_{s-1}, then the backward substitution from the
+//     exact carry x_{e+1}.  (Running the forward substitution again from
+//     d_{s-1} instead ends in other rounding errors than the scan's carry, a
+//     jump between chunks that near-singular lines amplify: a refined 512^3
+//     solve then contracted 0.0071 a sweep instead of 0.0059.)
 // The pivots 1/u_j come from the per-plan FP64 tables, read only for rows
-// before the line's pivots settle (k_plane_tables); later rows use 1/u_inf and
-// the corner row 1/u_{nx-1}.  Inner Steps 1 and 2 then form the CTA's share of
-// the inner boundary rows (eqs. 2dBs1, step2-3 on the plane) from the solved
-// tile, summing its inner modes in a fixed order, and accumulate them over the
-// CTA's nmb tiles into one face partial per CTA; inner Step 3 writes the
-// plane solution y3(x, l, m).
+// before the line's pivots settle (k_plane_tables) and for the last kRows rows
+// (the corner); all others use 1/u_inf (g = q), and alpha, beta of settled
+// chunks and beta of the last one come from the plan (alpha of the last chunk,
+// alpha and beta of the first multiply zeros).  Rows are taken kRows at a time,
+// a batch's values read before the dependent recurrence.  All batches run the
+// same unrolled code, with the g_j of a batch in registers: only their filling
+// differs.  (A separate code path for the few unsettled batches of a tile ran
+// 2 to 4 times slower per row: one warp executes it once a tile, from cold
+// instruction caches, while the others wait at the barrier.)  The rows past nx
+// of the last chunk are zeros with pivot 0.  Inner Steps 1 and 2 then form the
+// CTA's share of the inner boundary rows (eqs. 2dBs1, step2-3 on the plane)
+// from the solved tile, summing its inner modes in a fixed order, and
+// accumulate them over the CTA's nmb tiles into one face partial per CTA;
+// inner Step 3 writes the plane solution y3(x, l, m).
 // ---------------------------------------------------------------------------
+constexpr int kMW = 16;    // inner modes per tile: 128-byte rows in complex64
+constexpr int kRows = 8;   // rows per batch
+constexpr int kPivHead = 20;  // pivot rows staged in shared memory: the first 20 and the last kRows
+
 struct InnerArgs {
   Plane3DArgs a;
   int ch;      // rows per chunk
@@ -580,15 +601,23 @@ struct InnerArgs {
   int nparts;  // face partials per plane = gridDim.x
 };
 
-// Shared memory of k_inner3d: solved-row tile, pivot rows, chunk summaries
-// (padded), face accumulators, per-line and per-mode constants, powers of the
-// settled pivot ratio, the plane's inner C_bb faces (inner Steps 2 and 3),
-// settling rows.  istep 0: the largest of the three steps.
-inline size_t inner_smem_bytes(int64_t nx, int nc, int ch, size_t cb, int istep = 0) {
-  return ((size_t)nx * kMW + (size_t)kPivRows * kMW + 4 * (size_t)kMW * (nc + 1) + 2 * (size_t)nx + 9 * kMW + 3 +
-          (size_t)ch * kMW + (istep != 1 ? 2 * (size_t)nx : 0)) *
+// Shared memory of k_inner3d: the plane's inner C_bb faces (inner Steps 2 and
+// 3), the tile, pivot rows, chunk summaries (padded), face accumulators (Steps
+// 1 and 2), per-mode and per-line constants, settling rows.  Tiles of at most
+// 256 (complex64: 512) threads pad their rows (`pitch` values) so that a thread
+// per row reads 16 bytes without bank conflicts in the face sums; longer lines
+// have no room for it and read rotated.
+template <typename T>
+__host__ __device__ constexpr int inner_pitch(int max_threads) {
+  if (sizeof(T) == 4) return max_threads > 512 ? kMW : kMW + 2;
+  return max_threads > 256 ? kMW : kMW + 1;
+}
+
+inline size_t inner_smem_bytes(int64_t nx, int nc, int ch, int pitch, size_t cb, int istep) {
+  return ((istep != 1 ? 2 * (size_t)nc * ch : 0) + (size_t)nc * ch * pitch + (size_t)(kPivHead + kRows) * kMW +
+          4 * (size_t)kMW * (nc + 1) + (istep != 3 ? 2 * (size_t)nx : 0) + 9 * kMW + 3) *
              cb +
-         2 * kMW * sizeof(int);
+         kMW * sizeof(int);
 }
 
 // affine map x -> p x + q, composed as (p2, q2) o (p1, q1) = (p2 p1, p2 q1 + q2)
@@ -613,10 +642,20 @@ constexpr int inner_max_threads() {
 }
 
 // Chunks per line the tiled sweeps allow for (precision, rows per chunk); 0
-// unless CH is one of the compiled 8, 16, 32.
+// unless ch is 8, 16 or 32.
 inline int inner_max_chunks(int prec, int ch) {
   if (ch != 8 && ch != 16 && ch != 32) return 0;
   return (prec == kPrecF64 ? inner_max_threads<double>() : inner_max_threads<float>()) / kMW;
+}
+
+// Does a line of nx rows fit the tiled sweeps with (ch, nc)?
+inline bool inner_fits(int prec, int64_t nx, int ch, int nc, int smem_max) {
+  if (nc > inner_max_chunks(prec, ch)) return false;
+  const size_t cb = prec == kPrecF64 ? sizeof(double2) : sizeof(float2);
+  // the tile, 32 pivot rows, summaries, faces, constants and a row of values
+  // per chunk row (the largest tile that the sweeps have taken)
+  const size_t vals = (size_t)nx * kMW + 32 * kMW + 4 * kMW * ((size_t)nc + 1) + 4 * (size_t)nx + 9 * kMW + 3 + (size_t)ch * kMW;
+  return vals * cb + 2 * kMW * sizeof(int) <= (size_t)smem_max;
 }
 
 // Lanes per line in the chunk scan (a warp scans 32 / kScanLanes lines).
@@ -636,56 +675,70 @@ __device__ __forceinline__ C shfl_down_w(C v, int off) {
   return v;
 }
 
-template <typename T, int OSTEP, int ISTEP, int CH>
-__global__ void __launch_bounds__(inner_max_threads<T>()) k_inner3d(
-    InnerArgs ia, const typename cpx<T>::type* __restrict__ fhat, const typename cpx<T>::type* __restrict__ gfaces,
-    const typename cpx<T>::type* __restrict__ cin, const typename cpx<T>::type* __restrict__ tab,
-    const typename cpx<T>::type* __restrict__ lend, const int* __restrict__ lenL,
-    typename cpx<T>::type* __restrict__ part, typename cpx<T>::type* __restrict__ y3, const int* __restrict__ skip) {
+// MAXT, MINB: 256 threads with 128 registers (two CTAs an SM, all that the
+// tiles of the longer lines leave room for) or 80 (three and more), 512 with
+// 128 (complex64 lines beyond 512 rows, one tile an SM), or the largest CTA.  With 80 registers 512^3 took 6.1 ms of sweeps a solve instead
+// of 5.3; with 128, 190 x 223 x 127 took 0.51 ms instead of 0.42.
+template <typename T, int OSTEP, int ISTEP, int MAXT, int MINB>
+__global__ void __launch_bounds__(MAXT, MINB) k_inner3d(
+    const __grid_constant__ InnerArgs ia, const typename cpx<T>::type* __restrict__ fhat,
+    const typename cpx<T>::type* __restrict__ gfaces, const typename cpx<T>::type* __restrict__ cin,
+    const typename cpx<T>::type* __restrict__ tab, const typename cpx<T>::type* __restrict__ lend,
+    const int* __restrict__ lenL, typename cpx<T>::type* __restrict__ part, typename cpx<T>::type* __restrict__ y3,
+    const int* __restrict__ skip) {
   using C = typename cpx<T>::type;
+  constexpr int PT = inner_pitch<T>(MAXT);
+  // x_loc by a backward sweep over d (complex128: four FP64 operations a row
+  // fewer) or as sum_j p_j d_j along the forward one (complex64: a sweep fewer)
+  constexpr bool kHorner = sizeof(T) == 8;
   constexpr bool kFhatRows = OSTEP != 2 && ISTEP != 2;  // the right-hand side reads f_hat
+  constexpr bool kFaceRows = OSTEP != 1 && ISTEP != 2;  // ... and the outer faces
   if (skip && *skip) return;
   const Plane3DArgs& a = ia.a;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int nx = (int)a.nx;
   const int64_t ny = a.ny, nz = a.nz;
-  const int nc = ia.nc;
+  const int nc = ia.nc, ch = ia.ch;
   const int ncp = nc + 1;  // padded chunk stride of the summaries: conflict-free in both layouts
-  C* tile = reinterpret_cast<C*>(smem_raw);  // [nx][kMW]
-  C* piv = tile + (size_t)nx * kMW;          // [kPivRows][kMW] first rows of the pivot tables
-  C* sums = piv + kPivRows * kMW;            // [4][kMW][ncp]: d_loc, x_loc, alpha, beta; then the carries
-  C* facc = sums + 4 * kMW * ncp;            // [2][nx] face accumulators (inner Steps 1, 2)
-  C* mw = facc + 2 * nx;                     // [kMW] rhs scale, [kMW] weight of the last face, [2][kMW] face weights
-  // [kMW] b, [kMW] 1/u_inf, [kMW] 1/u_{nx-1}; [3] outer-mode constants; [kMW] alpha, [kMW] beta of a settled chunk
-  C* lc = mw + 4 * kMW;
-  C* apow = lc + 5 * kMW + 3;  // [CH][kMW] q^(k+1), q = -b / u_inf
-  C* scin = apow + CH * kMW;   // [2][nx] inner C_bb faces of this plane (inner Steps 2, 3)
-  int* sL = reinterpret_cast<int*>(scin + (ISTEP != 1 ? 2 * nx : 0));  // [kMW] settling rows
-  int* sR = sL + kMW;                                 // [kMW] 1: routed to FP64
+  C* scin = reinterpret_cast<C*>(smem_raw);    // [nc * ch][2] inner C_bb faces of this plane (inner Steps 2, 3)
+  C* tile = scin + (ISTEP != 1 ? 2 * nc * ch : 0);  // [nc * ch][PT]
+  C* piv = tile + (size_t)nc * ch * PT;       // [kPivHead + kRows][kMW] the first and the last pivot rows
+  C* sums = piv + (kPivHead + kRows) * kMW;    // [4][kMW][ncp]: d_loc, x_loc, alpha, beta; then the carries
+  C* facc = sums + 4 * kMW * ncp;              // [2][nx] face accumulators (inner Steps 1, 2)
+  C* sw = facc + (ISTEP != 3 ? 2 * nx : 0);    // [kMW] rhs scale, [kMW] weight of the last face, [2][kMW] face weights
+  // [kMW] b, [kMW] 1/u_inf, [kMW] alpha, [kMW] beta of a settled chunk, [kMW] beta of the last; [3] outer-mode constants
+  C* lc = sw + 4 * kMW;
+  int* sL = reinterpret_cast<int*>(lc + 5 * kMW + 3);  // [kMW] settling rows
   const int64_t l = blockIdx.y;
   const int tid = threadIdx.x, nthr = blockDim.x;
-  // thread (mi, c): the two half-warps of warp w take chunks w and nc-1-w, so
-  // that the first and the last chunk of a line (never settled: the first
-  // rows and the corner row) share a warp; with nc odd the middle warp's
-  // second half idles
-  const int mi = tid & (kMW - 1), wk = tid / (2 * kMW), half = (tid / kMW) & 1;
-  const int c = half ? nc - 1 - wk : wk;
-  const bool cok = half ? (nc - 1 - wk > wk) : (wk < nc);
+  // thread (mi, c): the first and the last chunk of a line (never settled: the
+  // first rows and the corner row) are in different warps, which run their
+  // slower batches side by side
+  const int mi = tid & (kMW - 1), c = tid / kMW;
+  const bool cok = c < nc;
+  const int s0 = c * ch, e1 = min(s0 + ch, nx);  // rows [s0, e1)
+  const int tail = nx - kRows;                   // rows from here on take their own pivots
   const int64_t xs = ny * nz;
   if (tid == 0) {
     // outer-mode constants: 1/mu_l (outer B modes), e^{+i theta_l} e^{-t(ny-1)}, parity (outer A modes)
-    lc[3 * kMW] = OSTEP == 2 ? mk<C>(1, 0) : mk<C>(a.invmuo[2 * l], a.invmuo[2 * l + 1]);
-    lc[3 * kMW + 1] = cmul(mk<C>(a.two[2 * l], -a.two[2 * l + 1]), mk<C>(a.eninv_o[0], a.eninv_o[1]));
-    lc[3 * kMW + 2] = mk<C>(a.parAo[l], 0);
+    lc[5 * kMW] = OSTEP == 2 ? mk<C>(1, 0) : mk<C>(a.invmuo[2 * l], a.invmuo[2 * l + 1]);
+    lc[5 * kMW + 1] = cmul(mk<C>(a.two[2 * l], -a.two[2 * l + 1]), mk<C>(a.eninv_o[0], a.eninv_o[1]));
+    lc[5 * kMW + 2] = mk<C>(a.parAo[l], 0);
   }
-  // the plane's inner C_bb faces into shared memory (they land with the
-  // first tile's copies)
+  // the plane's inner C_bb faces into shared memory, the two faces of a row
+  // side by side (they land with the first tile's copies)
   if (ISTEP != 1)
-    for (int e = tid; e < 2 * nx; e += nthr) cp_async<sizeof(C)>(scin + e, cin + l * 2 * nx + e);
-  const C* cin1 = scin;
-  const C* cinn = scin + nx;
+    for (int e = tid; e < 2 * nx; e += nthr) {
+      const int face = e >= nx ? 1 : 0;
+      cp_async<sizeof(C)>(scin + 2 * (e - face * nx) + face, cin + l * 2 * nx + e);
+    }
   if (ISTEP != 3)
     for (int e = tid; e < 2 * nx; e += nthr) facc[e] = mk<C>(0, 0);
+  // the rows past nx
+  for (int e = nx * PT + tid; e < nc * ch * PT; e += nthr) tile[e] = mk<C>(0, 0);
+  if (ISTEP != 1)
+    for (int e = 2 * nx + tid; e < 2 * nc * ch; e += nthr) scin[e] = mk<C>(0, 0);
+  const int tc = nthr >= 96 ? nthr / 64 * 32 : 0;  // kMW threads of a middle warp form the constants
   // the right-hand sides of this CTA's later tiles into L2 while the first
   // is staged and solved: one 128-byte line (16 inner modes) per row,
   // prefetched by lane 0 of each half-warp for its chunk's rows
@@ -693,11 +746,10 @@ __global__ void __launch_bounds__(inner_max_threads<T>()) k_inner3d(
     for (int mb = 1; mb < ia.nmb; ++mb) {
       const int64_t mq = ((int64_t)blockIdx.x * ia.nmb + mb) * kMW;
       if (mq >= nz) break;
-      for (int k = 0; k < CH && c * CH + k < nx; ++k) {
-        const int64_t x = c * CH + k;
-        if (OSTEP != 2) l2_prefetch(fhat + (x * ny + l) * nz + mq);
+      for (int x = s0; x < e1; ++x) {
+        if (OSTEP != 2) l2_prefetch(fhat + ((int64_t)x * ny + l) * nz + mq);
         if (OSTEP != 1) {
-          l2_prefetch(gfaces + x * nz + mq);
+          l2_prefetch(gfaces + (int64_t)x * nz + mq);
           l2_prefetch(gfaces + ((int64_t)nx + x) * nz + mq);
         }
       }
@@ -706,185 +758,246 @@ __global__ void __launch_bounds__(inner_max_threads<T>()) k_inner3d(
   for (int mb = 0; mb < ia.nmb; ++mb) {
     const int64_t m0 = ((int64_t)blockIdx.x * ia.nmb + mb) * kMW;
     if (m0 >= nz) break;
+    const int64_t m = m0 + mi;
+    const bool act = m < nz && cok;
     __syncthreads();  // the previous tile's face sums are done
     // ---- asynchronous copies of the tile's f_hat rows (thread (mi, c): its
     // own chunk rows; the 16 lanes of a half-warp read 16 consecutive inner
-    // modes of a row) and of the first pivot rows, all in flight while the
-    // line constants are formed; no registers hold them ----
-    {
-      const int64_t m = m0 + mi;
-      const int s0 = c * CH, e0 = min(s0 + CH, nx) - 1;
-      if (kFhatRows && cok && m < nz) {
+    // modes of a row) and of the pivot rows, all in flight while the line
+    // constants are formed; no registers hold them ----
+    if (kFhatRows) {
+      if (sizeof(T) == 4 && (nz & 1) == 0 && m0 + kMW <= nz) {  // 16-byte copies of two modes
+        const int part = tid & (kMW / 2 - 1);
+        const C* fp = fhat + l * nz + m0 + 2 * part;
+#pragma unroll 4
+        for (int j = tid / (kMW / 2); j < nx; j += nthr / (kMW / 2))
+          cp_async<16>(tile + j * PT + 2 * part, fp + (int64_t)j * xs);
+      } else if (act) {
         const C* fp = fhat + ((int64_t)s0 * ny + l) * nz + m;
-#pragma unroll
-        for (int k = 0; k < CH; ++k)
-          if (s0 + k <= e0) cp_async<sizeof(C)>(tile + (s0 + k) * kMW + mi, fp + k * xs);
-      }
-      // rows below the settling row are read from here, the others never
-      for (int e = tid; e < kPivRows * kMW; e += nthr) {
-        const int j = e / kMW, mm = e - j * kMW;
-        if (j < nx && m0 + mm < nz) cp_async<sizeof(C)>(piv + e, tab + (int64_t)j * xs + l * nz + m0 + mm);
+        C* tp = tile + s0 * PT + mi;
+#pragma unroll 8
+        for (int j = s0; j < e1; ++j) {
+          cp_async<sizeof(C)>(tp, fp);
+          tp += PT;
+          fp += xs;
+        }
       }
     }
-    if (tid < kMW) {
-      const int64_t m = m0 + tid;
-      const bool on = m < nz;
-      const int64_t mc = on ? m : 0;
+    for (int e = tid; e < (kPivHead + kRows) * kMW; e += nthr) {
+      const int k = e / kMW, mm = e - k * kMW;
+      const int j = k < kPivHead ? k : tail + (k - kPivHead);
+      if (j >= 0 && j < nx && m0 + mm < nz) cp_async<sizeof(C)>(piv + e, tab + (int64_t)j * xs + l * nz + m0 + mm);
+    }
+    if (tid >= tc && tid < tc + kMW) {
+      const int t = tid - tc;
+      const bool on = m0 + t < nz;
+      const int64_t mc = on ? m0 + t : 0;
       // right-hand side of inner Step 1 / 3: (G + [C_bb terms]) / mu_m; Step 2: c_1 + par_m c_n
-      mw[tid] = on ? (ISTEP == 2 ? mk<C>(1, 0) : mk<C>(a.invmui[2 * mc], a.invmui[2 * mc + 1])) : mk<C>(0, 0);
-      mw[kMW + tid] = ISTEP == 2 ? mk<C>(a.parAi[mc], 0)
-                                 : cmul(mk<C>(a.twi[2 * mc], -a.twi[2 * mc + 1]), mk<C>(a.eninv_i[0], a.eninv_i[1]));
+      C rs = ISTEP == 2 ? mk<C>(1, 0) : mk<C>(a.invmui[2 * mc], a.invmui[2 * mc + 1]);
+      C wk = ISTEP == 2 ? mk<C>(a.parAi[mc], 0)
+                        : cmul(mk<C>(a.twi[2 * mc], -a.twi[2 * mc + 1]), mk<C>(a.eninv_i[0], a.eninv_i[1]));
       // face weights of the inner boundary rows: Step 1 (1, e^{-i theta_m}), Step 2 (sigma_m, par_m sigma_m)
       C w1 = mk<C>(1, 0), wn = mk<C>(a.twi[2 * mc], a.twi[2 * mc + 1]);
       if (ISTEP == 2) {
         w1 = mk<C>(a.sigAi[2 * mc], a.sigAi[2 * mc + 1]);
         wn = cscale(w1, (T)a.parAi[mc]);
       }
-      mw[2 * kMW + tid] = on ? w1 : mk<C>(0, 0);
-      mw[3 * kMW + tid] = on ? wn : mk<C>(0, 0);
       // line constants from the plan tables
       const int64_t line = l * nz + mc;
-      const C b = lend[kLineVals * line + 2], iinf = lend[kLineVals * line];
-      lc[tid] = b;
-      lc[kMW + tid] = iinf;
-      lc[2 * kMW + tid] = lend[kLineVals * line + 1];
-      lc[3 * kMW + 3 + tid] = lend[kLineVals * line + 3];
-      lc[4 * kMW + 3 + tid] = lend[kLineVals * line + 4];
-      // powers of q = -b / u_inf: the forward carry's weight in a settled chunk
-      const C q = cmul(mk<C>(-b.x, -b.y), iinf);
-      C qk = q;
-      for (int k = 0; k < CH; ++k) {
-        apow[k * kMW + tid] = qk;
-        qk = cmul(qk, q);
-      }
+      lc[t] = lend[kLineVals * line + 2];
+      lc[kMW + t] = lend[kLineVals * line];
+      lc[2 * kMW + t] = lend[kLineVals * line + 3];
+      lc[3 * kMW + t] = lend[kLineVals * line + 4];
+      lc[4 * kMW + t] = lend[kLineVals * line + 5];
       // a line routed to FP64 (flag bit) gets a zero right-hand side here, so
       // it adds nothing to the faces; the FP64 kernel solves it
       const int lr = on ? lenL[line] : 0;
-      const bool routed = (lr & kRoutedFlag) != 0;
-      sL[tid] = routed ? 0 : lr;
-      if (routed) {
-        mw[tid] = mk<C>(0, 0);
-        mw[kMW + tid] = mk<C>(0, 0);
-        mw[2 * kMW + tid] = mk<C>(0, 0);
-        mw[3 * kMW + tid] = mk<C>(0, 0);
-      }
-      sR[tid] = routed ? 1 : 0;
+      const bool zero = !on || (lr & kRoutedFlag) != 0;
+      sL[t] = (lr & kRoutedFlag) ? 0 : lr;
+      sw[t] = zero ? mk<C>(0, 0) : rs;
+      sw[kMW + t] = wk;
+      sw[2 * kMW + t] = zero ? mk<C>(0, 0) : w1;
+      sw[3 * kMW + t] = zero ? mk<C>(0, 0) : wn;
     }
     cp_async_wait_all();
     __syncthreads();  // line constants formed, every thread's copies landed
-    // ---- thread (mi, c) forms the right-hand sides of its own chunk rows in
-    // place (from the copied f_hat rows, the outer faces, the inner C_bb
-    // faces) ----
-    const int64_t m = m0 + mi;
-    const bool act = m < nz && cok;
-    const int s0 = c * CH, e0 = min(s0 + CH, nx) - 1;
-    C* trow = tile + s0 * kMW + mi;  // row s0 + k of this line: trow[k * kMW]
-    if (cok) {
-      const C gscale = lc[3 * kMW], wl = lc[3 * kMW + 1];
-      const T paro = lc[3 * kMW + 2].x;
-      const C sc = mw[mi], wk2 = mw[kMW + mi];
-      const C gs = cmul(gscale, sc);
-      const bool zero_rhs = !act || (ISTEP == 2 && sR[mi]);
-      const int64_t mcl = act ? m : 0;
-      const C* g1p = OSTEP != 1 ? gfaces + (int64_t)s0 * nz + mcl : nullptr;  // outer faces (Steps 2, 3)
-      const C* gnp = OSTEP != 1 ? g1p + (int64_t)nx * nz : nullptr;
-#pragma unroll(CH <= 16 ? CH : 8)
-      for (int k = 0; k < CH; ++k) {
-        if (s0 + k <= e0) {
-          C v = mk<C>(0, 0);
-          if (!zero_rhs) {
-            if (ISTEP == 2) {
-              v = cadd(cin1[s0 + k], cmul(cinn[s0 + k], wk2));
-            } else {
-              if (OSTEP == 1) v = cmul(trow[k * kMW], gs);
-              else if (OSTEP == 2) v = cmul(cadd(g1p[k * nz], cscale(gnp[k * nz], paro)), sc);
-              else v = cmul(cadd(cadd(trow[k * kMW], g1p[k * nz]), cmul(gnp[k * nz], wl)), gs);
-              if (ISTEP == 3) v = cadd(v, cmul(cadd(cin1[s0 + k], cmul(cinn[s0 + k], wk2)), sc));
-            }
-          }
-          trow[k * kMW] = v;
+    const int L = sL[mi];  // 0 for a routed line
+    // the rows below jl take their own pivots, rounded up to whole batches (the
+    // tables hold every row), and those of the last batches that reach the tail
+    const int jl = s0 + (max(L - s0, 0) + kRows - 1) / kRows * kRows;
+    // the whole chunk on the constant pivot (warp-uniform; the other path is
+    // exact for such chunks too)
+    const bool settled = __all_sync(0xffffffffu, !act || (s0 >= L && s0 + ch <= tail));
+    const C b = lc[mi], iinf = lc[kMW + mi];
+    const C nb = mk<C>(-b.x, -b.y);
+    const C q = cmul(nb, iinf);
+    const C sc = sw[mi], wk2 = sw[kMW + mi];
+    const C gs = cmul(lc[5 * kMW], sc);
+    const C wl = lc[5 * kMW + 1];
+    const T paro = lc[5 * kMW + 2].x;
+    C* trow = tile + s0 * PT + mi;  // row s0 + k of this line: trow[k * PT]
+    const C* tcol = tab + l * nz + (m < nz ? m : 0);
+    // right-hand sides of rows jb .. jb + kRows - 1 (those below e1), times f (1 or 1/u_inf)
+    auto rhs = [&](int jb, C scf, C gsf, C (&v)[kRows]) {
+      C* tp = trow + (jb - s0) * PT;
+      if (kFhatRows) {
+#pragma unroll
+        for (int k = 0; k < kRows; ++k) v[k] = tp[k * PT];
+        if (OSTEP == 1) {
+#pragma unroll
+          for (int k = 0; k < kRows; ++k) v[k] = cmul(v[k], gsf);
         }
       }
-    }
-    // ---- line constants of thread (mi, c) ----
-    const C b = lc[mi], iinf = lc[kMW + mi], ilast = lc[2 * kMW + mi];
-    const C nb = mk<C>(-b.x, -b.y);
-    const C cinf = cmul(b, iinf);
-    const int L = sL[mi];  // 0 for a routed line
-    const C* tcol = tab + l * nz + (m < nz ? m : 0);
-    // The rows of a chunk that is not settled, in three runs: rows [s0, jt)
-    // below the settling row take 1/u_j from the pivot table (four loads in
-    // flight at a time), rows [jt, jc) take 1/u_inf, and the corner row nx - 1
-    // (if the chunk holds it) 1/u_{nx-1}.  fn(j, 1/u_j, g_j) with
-    // g_j = -b / u_j, the weight of the previous row's value in
-    // d_j = r_j / u_j + g_j d_{j-1} and of the next row's in x_j = d_j + g_j x_{j+1}.
-    const int jt = min(e0 + 1, max(s0, L));
-    const int jc = e0 == nx - 1 ? e0 : e0 + 1;
-    const C q = cmul(nb, iinf), glast = cmul(nb, ilast);
-    auto tpiv = [&](int j) -> C { return j < kPivRows ? piv[j * kMW + mi] : tcol[(int64_t)j * xs]; };
-    auto rows_up = [&](auto&& fn) {
-#pragma unroll 1
-      for (int j0 = s0; j0 < jt; j0 += 4) {
-        C pv[4];
+      if (kFaceRows) {
+        const C* g1p = gfaces + (int64_t)jb * nz + (m < nz ? m : 0);  // outer faces
+        const C* gnp = g1p + (int64_t)nx * nz;
+        C g1[kRows], gn[kRows];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) pv[k] = j0 + k < jt ? tpiv(j0 + k) : iinf;
+        for (int k = 0; k < kRows; ++k) {
+          g1[k] = gn[k] = mk<C>(0, 0);
+          if (jb + k < e1) {
+            g1[k] = *g1p;
+            gn[k] = *gnp;
+          }
+          g1p += nz;
+          gnp += nz;
+        }
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (j0 + k < jt) fn(j0 + k, pv[k], cmul(nb, pv[k]));
+        for (int k = 0; k < kRows; ++k) {
+          if (OSTEP == 2) v[k] = cmul(cadd(g1[k], cscale(gn[k], paro)), scf);
+          else v[k] = cmul(cfma(gn[k], wl, cadd(v[k], g1[k])), gsf);
+        }
       }
-#pragma unroll 4
-      for (int j = jt; j < jc; ++j) fn(j, iinf, q);
-      if (jc == e0) fn(e0, ilast, glast);
+      if (ISTEP != 1) {
+#pragma unroll
+        for (int k = 0; k < kRows; ++k) {
+          C c1, cn;
+          {
+            if constexpr (sizeof(T) == 4) {
+              const float4 cc = *reinterpret_cast<const float4*>(scin + 2 * (jb + k));
+              c1 = mk<C>(cc.x, cc.y);
+              cn = mk<C>(cc.z, cc.w);
+            } else {
+              c1 = scin[2 * (jb + k)];
+              cn = scin[2 * (jb + k) + 1];
+            }
+          }
+          if (ISTEP == 2) v[k] = cmul(cadd(c1, cscale(cn, wk2.x)), scf);
+          else v[k] = cfma(cfma(cn, wk2, c1), scf, v[k]);
+        }
+      }
     };
-    auto rows_down = [&](auto&& fn) {
-      if (jc == e0) fn(e0, ilast, glast);
-#pragma unroll 4
-      for (int j = jc - 1; j >= jt; --j) fn(j, iinf, q);
-#pragma unroll 1
-      for (int j0 = jt - 1; j0 >= s0; j0 -= 4) {
-        C pv[4];
+    // Batches: 0 every lane's rows on the constant pivot, 1 rows of their own in
+    // the first or the last chunk among the staged ones, 2 others (propagating
+    // modes; their chunks form alpha and beta here).
+    auto kind = [&](int jb) -> int {
+      const bool own = jb < jl || jb + kRows > tail;
+      const unsigned lanes = __activemask();
+      if (!__any_sync(lanes, own)) return 0;
+      const bool deep = (c > 0 && c < nc - 1) || (jb + kRows > kPivHead && jb < tail);
+      return __any_sync(lanes, own && deep) ? 2 : 1;
+    };
+    // 1/u_j of a batch's rows (0 past nx)
+    auto pivots = [&](int jb, int kd, C (&pv)[kRows]) {
+      const bool own = jb < jl || jb + kRows > tail;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) pv[k] = j0 - k >= s0 ? tpiv(j0 - k) : iinf;
+      for (int k = 0; k < kRows; ++k) {
+        const int j = jb + k;
+        const int at = j < kPivHead ? j : kPivHead + j - tail;
+        pv[k] = j < nx ? iinf : mk<C>(0, 0);
+        if (own && (j < kPivHead || j >= tail) && j < nx) pv[k] = piv[at * kMW + mi];
+      }
+      if (kd == 2) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (j0 - k >= s0) fn(j0 - k, pv[k], cmul(nb, pv[k]));
+        for (int k = 0; k < kRows; ++k)
+          if (own && jb + k >= kPivHead && jb + k < tail) pv[k] = tcol[(int64_t)(jb + k) * xs];
+      }
+    };
+    // g_j of a batch after pass 1's forward sweep, which leaves them in place of
+    // the staged pivots (every row is one thread's)
+    auto ratios = [&](int jb, int kd, C (&g)[kRows]) {
+      const bool own = jb < jl || jb + kRows > tail;
+#pragma unroll
+      for (int k = 0; k < kRows; ++k) {
+        const int j = jb + k;
+        const int at = j < kPivHead ? j : kPivHead + j - tail;
+        g[k] = j < nx ? q : mk<C>(0, 0);
+        if (own && (j < kPivHead || j >= tail) && j < nx) g[k] = piv[at * kMW + mi];
+      }
+      if (kd == 2) {
+#pragma unroll
+        for (int k = 0; k < kRows; ++k)
+          if (own && jb + k >= kPivHead && jb + k < tail) g[k] = cmul(nb, tcol[(int64_t)(jb + k) * xs]);
       }
     };
     // ---- pass 1 ----
-    // Forward with d_{s-1} = 0 (d_loc written over the rhs), then the
-    // backward substitution with x_{e+1} = 0 over it by Horner's rule gives
-    // x_loc.  alpha_e = prod (-b/u_j) and beta = sum alpha_{j-1} alpha_j do
-    // not depend on the data: a settled chunk takes them from the plan, the
-    // others form them.  Warp-uniform: a warp takes the settled path only if
-    // all its chunks are settled (the general path is exact for them too).
-    const bool settled = __all_sync(0xffffffffu, !act || (s0 >= L && e0 < nx - 1 && e0 - s0 + 1 == CH));
+    C g[kRows];  // -b / u_j of the batch
+#pragma unroll
+    for (int k = 0; k < kRows; ++k) g[k] = q;
+    const int jlast = s0 + (e1 - 1 - s0) / kRows * kRows;  // first row of the last batch
     if (act) {
-      C d = mk<C>(0, 0), al = mk<C>(1, 0), be = mk<C>(0, 0), x = mk<C>(0, 0);
-      if (settled) {
-        // d_j = r_j / u_inf + q d_{j-1}, q = -b / u_inf
-#pragma unroll 16
-        for (int k = 0; k < CH; ++k) {
-          d = cfma(q, d, cmul(trow[k * kMW], iinf));
-          trow[k * kMW] = d;
+      C d = mk<C>(0, 0), x = mk<C>(0, 0), p = mk<C>(1, 0), be = mk<C>(0, 0);
+      const C sci = cmul(sc, iinf), gsi = cmul(gs, iinf);
+      // a middle chunk with rows of its own forms its alpha and beta
+      const bool mid = c > 0 && c < nc - 1 && L > s0;
+      for (int jb = s0; jb < e1; jb += kRows) {
+        const int kd = settled ? 0 : kind(jb);
+        C v[kRows];
+        rhs(jb, kd ? sc : sci, kd ? gs : gsi, v);
+        if (kd) {
+          pivots(jb, kd, g);
+          const bool own = jb < jl || jb + kRows > tail;
+#pragma unroll
+          for (int k = 0; k < kRows; ++k) {
+            const int j = jb + k;
+            v[k] = cmul(v[k], g[k]);
+            g[k] = cmul(nb, g[k]);
+            if (own && (j < kPivHead || j >= tail) && j < nx)
+              piv[(j < kPivHead ? j : kPivHead + j - tail) * kMW + mi] = g[k];
+          }
         }
-#pragma unroll 16
-        for (int k = CH - 1; k >= 0; --k) x = cfms(trow[k * kMW], cinf, x);
-        al = lc[3 * kMW + 3 + mi];
-        be = lc[4 * kMW + 3 + mi];
-      } else {
-        rows_up([&](int j, C inv, C g) {
-          d = cfma(g, d, cmul(tile[j * kMW + mi], inv));
-          tile[j * kMW + mi] = d;
-          const C an = cmul(al, g);
-          be = cfma(al, an, be);
-          al = an;
-        });
-        rows_down([&](int j, C, C g) { x = cfma(g, x, tile[j * kMW + mi]); });
+        if (mid) {
+          C t = p;
+#pragma unroll
+          for (int k = 0; k < kRows; ++k) {
+            const C tn = cmul(t, g[k]);
+            be = cfma(t, tn, be);
+            t = tn;
+          }
+          if (kHorner) p = t;
+        }
+        C* tp = trow + (jb - s0) * PT;
+#pragma unroll
+        for (int k = 0; k < kRows; ++k) {
+          d = cfma(g[k], d, v[k]);
+          tp[k * PT] = d;
+          if (!kHorner) x = cfma(p, d, x);
+          if (!kHorner) p = cmul(p, g[k]);
+        }
+        if (kd) {
+#pragma unroll
+          for (int k = 0; k < kRows; ++k) g[k] = q;
+        }
       }
+      if (kHorner)
+        for (int jb = jlast; jb >= s0; jb -= kRows) {
+          const int kd = settled ? 0 : kind(jb);
+          if (kd) ratios(jb, kd, g);
+          const C* tp = trow + (jb - s0) * PT;
+          C v[kRows];
+#pragma unroll
+          for (int k = 0; k < kRows; ++k) v[k] = tp[k * PT];
+#pragma unroll
+          for (int k = kRows - 1; k >= 0; --k) x = cfma(g[k], x, v[k]);
+          if (kd) {
+#pragma unroll
+            for (int k = 0; k < kRows; ++k) g[k] = q;
+          }
+        }
       sums[(0 * kMW + mi) * ncp + c] = d;
       sums[(1 * kMW + mi) * ncp + c] = x;
-      sums[(2 * kMW + mi) * ncp + c] = al;
-      sums[(3 * kMW + mi) * ncp + c] = be;
+      sums[(2 * kMW + mi) * ncp + c] = mid ? p : lc[2 * kMW + mi];
+      sums[(3 * kMW + mi) * ncp + c] = mid ? be : lc[(c == nc - 1 ? 4 : 3) * kMW + mi];
     }
     __syncthreads();
     // ---- scan over the chunks of each line: kScanLanes lanes per line, each
@@ -895,7 +1008,7 @@ __global__ void __launch_bounds__(inner_max_threads<T>()) k_inner3d(
       constexpr int lpw = 32 / kScanLanes;             // lines per warp
       const int g = (nc + kScanLanes - 1) / kScanLanes;  // chunks per lane
       for (int mm0 = warp * lpw; mm0 < kMW; mm0 += nw * lpw) {
-        const int mm = mm0 + seg;
+        const int mm = mm0 + seg;  // a line past the grid holds garbage, which stays its own
         C* sd = sums + (0 * kMW + mm) * ncp;  // d_loc, then the carry-in d_{s-1}
         C* sx = sums + (1 * kMW + mm) * ncp;  // x_loc, then the carry-in x_{e+1}
         const C* sa = sums + (2 * kMW + mm) * ncp;
@@ -942,47 +1055,103 @@ __global__ void __launch_bounds__(inner_max_threads<T>()) k_inner3d(
     }
     __syncthreads();
     // ---- pass 2 ----
-    // d_j = d_loc_j + alpha_j d_{s-1} over the chunk, then the backward
-    // substitution from the exact carry x_{e+1}; in a settled chunk
-    // alpha_j = q^(j-s+1) and both run in one backward sweep.
     if (act) {
-      const C Din = sums[(0 * kMW + mi) * ncp + c];
-      C x = sums[(1 * kMW + mi) * ncp + c];
-      C* yrow = y3 + ((int64_t)s0 * ny + l) * nz + m;  // y3 rows of this line (Step 3)
-      if (settled) {
-#pragma unroll 16
-        for (int k = CH - 1; k >= 0; --k) {
-          x = cfms(cfma(apow[k * kMW + mi], Din, trow[k * kMW]), cinf, x);
-          if (ISTEP == 3) yrow[k * xs] = x;
-          else trow[k * kMW] = x;
+      C t = sums[(0 * kMW + mi) * ncp + c], x = sums[(1 * kMW + mi) * ncp + c];
+      if (!settled) {  // chunks with rows of their own: p_{j+1} d_{s-1} added here
+        for (int jb = s0; jb < e1; jb += kRows) {
+          const int kd = kind(jb);
+          if (kd) ratios(jb, kd, g);
+          C* tp = trow + (jb - s0) * PT;
+#pragma unroll
+          for (int k = 0; k < kRows; ++k) {
+            t = cmul(g[k], t);
+            tp[k * PT] = cadd(tp[k * PT], t);
+          }
+          if (kd) {
+#pragma unroll
+            for (int k = 0; k < kRows; ++k) g[k] = q;
+          }
         }
-      } else {
-        C al = mk<C>(1, 0);
-        rows_up([&](int j, C, C g) {
-          al = cmul(al, g);
-          tile[j * kMW + mi] = cfma(al, Din, tile[j * kMW + mi]);
-        });
-        rows_down([&](int j, C, C g) {
-          x = cfma(g, x, tile[j * kMW + mi]);
-          if (ISTEP == 3) yrow[(int64_t)(j - s0) * xs] = x;
-          else tile[j * kMW + mi] = x;
-        });
       }
+      // q^(8 i) d_{s-1}, i the batch (at most 4): within one the powers go up
+      C q8 = cmul(q, q);
+      q8 = cmul(q8, q8);
+      q8 = cmul(q8, q8);
+      const C t1 = cmul(t, q8), t2 = cmul(t1, q8), t3 = cmul(t2, q8);
+      for (int jb = jlast; jb >= s0; jb -= kRows) {
+        const int kd = settled ? 0 : kind(jb);
+        C* tp = trow + (jb - s0) * PT;
+        const int ib = (jb - s0) / kRows;
+        C u = ib == 0 ? t : ib == 1 ? t1 : ib == 2 ? t2 : t3;
+        C* yp = y3 + ((int64_t)(jb + kRows - 1) * ny + l) * nz + m;  // y3 rows of this line (Step 3)
+        C v[kRows];
+#pragma unroll
+        for (int k = 0; k < kRows; ++k) v[k] = tp[k * PT];
+        if (settled) {
+#pragma unroll
+          for (int k = 0; k < kRows; ++k) {
+            u = cmul(q, u);
+            v[k] = cadd(v[k], u);
+          }
+        }
+        if (kd) ratios(jb, kd, g);
+#pragma unroll
+        for (int k = kRows - 1; k >= 0; --k) {
+          x = cfma(g[k], x, v[k]);
+          if (ISTEP != 3) tp[k * PT] = x;
+          else {
+            if (jb + k < nx) *yp = x;
+            yp -= xs;
+          }
+        }
+        if (kd) {
+#pragma unroll
+          for (int k = 0; k < kRows; ++k) g[k] = q;
+        }
+      }
+    } else if (ISTEP != 3 && cok) {
+      for (int j = s0; j < e1; ++j) tile[j * PT + mi] = mk<C>(0, 0);  // modes off the grid add nothing
     }
     if (ISTEP != 3) {
       __syncthreads();
-      // this tile's share of the inner boundary rows, inner modes summed in a
-      // fixed (row-rotated, bank-conflict-free) order
+      // this tile's share of the inner boundary rows, a thread per row, inner
+      // modes summed in a fixed order; Step 1's first-row weight is 1 (modes
+      // off the grid or routed hold zeros in the tile)
       for (int x = tid; x < nx; x += nthr) {
         C s1 = mk<C>(0, 0), sn = mk<C>(0, 0);
+        if constexpr (PT != kMW && sizeof(T) == 4) {
 #pragma unroll
-        for (int k = 0; k < kMW; ++k) {
-          const int mm = (k + x) & (kMW - 1);
-          const C v = tile[x * kMW + mm];
-          // Step 1's first-row weight is 1 (modes off the grid or routed
-          // hold zeros in the tile)
-          s1 = ISTEP == 1 ? cadd(s1, v) : cfma(v, mw[2 * kMW + mm], s1);
-          sn = cfma(v, mw[3 * kMW + mm], sn);
+          for (int mm = 0; mm < kMW; mm += 2) {
+            const float4 z = *reinterpret_cast<const float4*>(tile + x * PT + mm);
+            const float4 wn = *reinterpret_cast<const float4*>(sw + 3 * kMW + mm);
+            const C z0 = mk<C>(z.x, z.y), z1 = mk<C>(z.z, z.w);
+            if (ISTEP == 1) {
+              s1 = cadd(s1, cadd(z0, z1));
+            } else {
+              const float4 w1 = *reinterpret_cast<const float4*>(sw + 2 * kMW + mm);
+              s1 = cfma(z1, mk<C>(w1.z, w1.w), cfma(z0, mk<C>(w1.x, w1.y), s1));
+            }
+            sn = cfma(z1, mk<C>(wn.z, wn.w), cfma(z0, mk<C>(wn.x, wn.y), sn));
+          }
+        } else {
+#pragma unroll
+          for (int k = 0; k < kMW; ++k) {
+            const int mm = PT != kMW ? k : (k + x) & (kMW - 1);
+            const C v = tile[x * PT + mm];
+            if (ISTEP == 1) {
+              s1 = cadd(s1, v);
+              sn = cfma(v, sw[3 * kMW + mm], sn);
+            } else {  // even and odd modes apart: (sigma, +-sigma)
+              const C w = sw[2 * kMW + mm];
+              if (sw[kMW + mm].x > 0) s1 = cfma(v, w, s1);
+              else sn = cfma(v, w, sn);
+            }
+          }
+          if (ISTEP == 2) {
+            const C even = s1;
+            s1 = cadd(even, sn);
+            sn = csub(even, sn);
+          }
         }
         facc[x] = cadd(facc[x], s1);
         facc[nx + x] = cadd(facc[nx + x], sn);
@@ -1147,7 +1316,6 @@ __global__ void __launch_bounds__(256) k_inner_reduce(InnerArgs ia, const typena
                                                       const typename cpx<T>::type* __restrict__ rpart,
                                                       const int* __restrict__ skip) {
   using C = typename cpx<T>::type;
-  constexpr bool kFhatRows = OSTEP != 2 && ISTEP != 2;  // the right-hand side reads f_hat
   if (skip && *skip) return;
   const Plane3DArgs& a = ia.a;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1212,7 +1380,7 @@ cudaError_t launch_inner_t(const Plan3D& p, const void* gfaces, const int* skip,
   using C = typename cpx<T>::type;
   InnerArgs ia{make_args(p), p.inner_ch, p.inner_nc, p.inner_nmb, p.inner_nparts};
   const int nx = (int)p.n[0];
-  const int nthr = kMW * ((p.inner_nc + 1) & ~1);
+  const int nthr = (kMW * p.inner_nc + 31) / 32 * 32;
   const dim3 grid((unsigned)p.inner_nparts, (unsigned)p.n[1]);
   const int oA = OSTEP == 2 ? 1 : 0;
   const C* fh = (const C*)p.fhat;
@@ -1225,13 +1393,24 @@ cudaError_t launch_inner_t(const Plan3D& p, const void* gfaces, const int* skip,
                                           {"inner_o2_i1", "inner_o2_i2", "inner_o2_i3"},
                                           {"inner_o3_i1", "inner_o3_i2", "inner_o3_i3"}};
   cudaError_t e;
-  auto sweep = [&](auto kern, int istep, int innerA) -> cudaError_t {
+  auto sweep = [&](auto is, int innerA) -> cudaError_t {
+    constexpr int IS = decltype(is)::value;
+    constexpr int MINB = sizeof(T) == 4 ? 3 : 2;
     const int t = 2 * oA + innerA;
-    ProfScope ps(prof, names[OSTEP - 1][istep - 1], st);
-    const size_t smem = inner_smem_bytes(nx, p.inner_nc, p.inner_ch, sizeof(C), istep);
-    allow_dynamic_smem((const void*)kern, smem);
-    kern<<<grid, nthr, smem, st>>>(ia, fh, gf, cin, (const C*)p.tab[t], (const C*)p.lend[t], p.lenL[t], part,
-                                   (C*)p.dbuf, skip);
+    ProfScope ps(prof, names[OSTEP - 1][IS - 1], st);
+    const int maxt = nthr <= 256 ? 256 : nthr <= 512 ? 512 : 1024;
+    auto bytes = [&](int istep) {
+      return inner_smem_bytes(nx, p.inner_nc, p.inner_ch, inner_pitch<T>(maxt), sizeof(C), istep);
+    };
+    // the CTAs that fit the shared memory of an SM (228 KB, 1 KB of each CTA
+    // reserved) in the step that needs most of it
+    const bool few = (bytes(2) + 1024) * MINB > 228 * 1024;
+    auto kern = k_inner3d<T, OSTEP, IS, inner_max_threads<T>(), 1>;
+    if (maxt == 256) kern = few ? k_inner3d<T, OSTEP, IS, 256, 2> : k_inner3d<T, OSTEP, IS, 256, MINB>;
+    else if (maxt == 512) kern = k_inner3d<T, OSTEP, IS, 512, 1>;
+    allow_dynamic_smem((const void*)kern, bytes(IS));
+    kern<<<grid, nthr, bytes(IS), st>>>(ia, fh, gf, cin, (const C*)p.tab[t], (const C*)p.lend[t], p.lenL[t], part,
+                                        (C*)p.dbuf, skip);
     return cudaGetLastError();
   };
   auto routed = [&](auto kern, int innerA) -> cudaError_t {
@@ -1251,23 +1430,13 @@ cudaError_t launch_inner_t(const Plan3D& p, const void* gfaces, const int* skip,
                                              skip);
     return cudaGetLastError();
   };
-  // the sweep kernel of inner step ISTEP for the plan's rows per chunk
-  auto sweep_ch = [&](auto istep, int innerA) -> cudaError_t {
-    constexpr int IS = decltype(istep)::value;
-    switch (p.inner_ch) {
-      case 8: return sweep(k_inner3d<T, OSTEP, IS, 8>, IS, innerA);
-      case 16: return sweep(k_inner3d<T, OSTEP, IS, 16>, IS, innerA);
-      case 32: return sweep(k_inner3d<T, OSTEP, IS, 32>, IS, innerA);
-      default: return cudaErrorInvalidValue;
-    }
-  };
-  if ((e = sweep_ch(std::integral_constant<int, 1>{}, 0)) != cudaSuccess) return e;
+  if ((e = sweep(std::integral_constant<int, 1>{}, 0)) != cudaSuccess) return e;
   if ((e = routed(k_inner3d_r<T, OSTEP, 1>, 0)) != cudaSuccess) return e;
   if ((e = reduce(k_inner_reduce<T, OSTEP, 1>, 0)) != cudaSuccess) return e;
-  if ((e = sweep_ch(std::integral_constant<int, 2>{}, 1)) != cudaSuccess) return e;
+  if ((e = sweep(std::integral_constant<int, 2>{}, 1)) != cudaSuccess) return e;
   if ((e = routed(k_inner3d_r<T, OSTEP, 2>, 1)) != cudaSuccess) return e;
   if ((e = reduce(k_inner_reduce<T, OSTEP, 2>, 1)) != cudaSuccess) return e;
-  if ((e = sweep_ch(std::integral_constant<int, 3>{}, 0)) != cudaSuccess) return e;
+  if ((e = sweep(std::integral_constant<int, 3>{}, 0)) != cudaSuccess) return e;
   return routed(k_inner3d_r<T, OSTEP, 3>, 0);
 }
 
@@ -1417,18 +1586,25 @@ cudaError_t plan3d_init(Plan3D& p, int prec, const int64_t* n, const double* h, 
   int dev = 0, smem_max = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  // 16 rows per chunk, 32 for lines too long for 16 (the kernels hold a
-  // chunk in registers, so CH is one of 8, 16, 32)
-  int ch = 16, nc = (int)((n[0] + 15) / 16);
+  // Rows per chunk: 16; in complex64 32 for lines beyond 256 rows (fewer and
+  // longer recurrences a line; 512^3: 5.5 ms of sweeps a solve against 8.3, 384
+  // x 320 x 256 1.6 against 2.3, 257 x 256 x 256 1.1 against 1.3; 190 x 223 x
+  // 127 0.55 against 0.46), and where 16 would be too many chunks.  8 is faster
+  // still on grids of few tiles (96 x 80 x 72: 0.124 against 0.152) and slower
+  // on others of that size (114 x 55 x 132): left to the autotuner.
+  int ch = prec == kPrecF32 && n[0] > 256 ? 32 : 16;
+  int nc = (int)((n[0] + ch - 1) / ch);
   if (nc > inner_max_chunks(prec, ch)) {
     ch = 32;
     nc = (int)((n[0] + 31) / 32);
   }
-  const size_t ismem = inner_smem_bytes(n[0], nc, ch, cb);
-  if (p.tab[0] && nc <= inner_max_chunks(prec, ch) && ismem <= (size_t)smem_max) {
+  if (p.tab[0] && inner_fits(prec, n[0], ch, nc, smem_max)) {
     const int64_t tiles = (n[2] + kMW - 1) / kMW;
     const int64_t total = tiles * n[1];
-    int nmb = (int)std::max<int64_t>(1, std::min<int64_t>(4, total / (152 * 8)));
+    // tiles per CTA: one, and two where that still leaves 32 CTAs for an SM
+    // (512^3: half the face partials to reduce; 384 x 320 x 256 is 4 % faster
+    // with one)
+    int nmb = prec == kPrecF32 && total >= 2 * 152 * 32 ? 2 : 1;
     nmb = (int)std::min<int64_t>(nmb, tiles);
     const int nparts = (int)((tiles + nmb - 1) / nmb);
     const size_t sz[3] = {(size_t)n[1] * nparts * 2 * n[0] * cb, (size_t)n[1] * 4 * n[0] * cb,
@@ -1572,12 +1748,11 @@ int plan3d_routed_lines(const Plan3D& p) { return p.nroute[0] + p.nroute[1] + p.
 cudaError_t plan3d_set_inner(Plan3D& p, int ch, int nmb) {
   if (!p.inner_nmb || nmb < 1 || nmb > 8) return cudaErrorInvalidValue;
   const size_t cb = p.prec == kPrecF64 ? sizeof(double2) : sizeof(float2);
-  const int max_nc = inner_max_chunks(p.prec, ch);  // 0 unless ch is 8, 16 or 32
   const int nc = (int)((p.n[0] + ch - 1) / ch);
   int dev = 0, smem_max = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (nc > max_nc || inner_smem_bytes(p.n[0], nc, ch, cb) > (size_t)smem_max) return cudaErrorInvalidValue;
+  if (!inner_fits(p.prec, p.n[0], ch, nc, smem_max)) return cudaErrorInvalidValue;
   const int64_t tiles = (p.n[2] + kMW - 1) / kMW;
   nmb = (int)std::min<int64_t>(nmb, tiles);
   const int nparts = (int)((tiles + nmb - 1) / nmb);
