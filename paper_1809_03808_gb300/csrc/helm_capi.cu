@@ -448,37 +448,40 @@ int solve2d_core(helm_plan* p, const void* in, int in_is_double, void* out, int 
   const void* sco = f64 ? (const void*)ax.sc_out : (const void*)ax.sc_out32;
   const double one[2] = {1.0, 0.0}, inv_n1[2] = {1.0 / (double)n1, 0.0};
   const double en_n1[2] = {ax.en[0] / (double)n1, ax.en[1] / (double)n1};
-  const int64_t nparts = (n1 + 127) / 128;  // face partials: one per block of 128 lines
+  // face partials: one per block of lines of the step kernels
+  const int64_t lpb = p->tabB && f64 ? tri2d_tab_lines(n1, a.nchunks) : 128;
+  const int64_t nparts = (n1 + lpb - 1) / lpb;
   HELM_PK("dft_fwd", launch_dft_rows(prec, in, in_is_double, p->fhat, fhat_mode, nx, ax.dft, tw, -1, 1.0, 0.0, sci,
                                      nullptr, skip, st, p->dev_err));
   if (dbg_fhat) HELM_CK(cudaMemcpyAsync(dbg_fhat, p->fhat, nx * n1 * cb, cudaMemcpyDeviceToDevice, st));
   // a2: Step 1
   if (p->tabB && prec == kPrecF64)
-    HELM_CK(launch_tri2d_tab(1, p->fhat, nullptr, p->tabB, p->rec, nullptr, p->partial, a, skip, st, p->prof.on ? &p->prof : nullptr));
+    HELM_CK(launch_tri2d_tab(1, p->fhat, nullptr, p->tabB, p->rec, nullptr, p->partial, a, skip, st, p->prof.on ? &p->prof : nullptr,
+                             p->constB));
   else if (p->tabB)
     HELM_CK(launch_tri2d_t32(1, p->fhat, nullptr, p->tabB, p->rec, nullptr, p->partial, a, skip, st, p->prof.on ? &p->prof : nullptr,
                              p->constB, p->dev_err));
   else
     HELM_CK(launch_tri2d(prec, 1, p->fhat, nullptr, p->ustartB, p->rec, nullptr, p->partial, a, skip, st, p->prof.on ? &p->prof : nullptr, p->constB));
-  HELM_PK("reduce_faces", launch_reduce_faces(prec, p->partial, fv, nx, nparts, inv_n1, en_n1, skip, st));
+  HELM_PK("faces_cbb", launch_faces_cbb(prec, p->partial, nparts, inv_n1, en_n1, fv, nullptr, fc, nx, p->h[0], p->h[1],
+                                        p->wc[0], p->wc[1], p->omega * p->omega, ax.g, ax.ginv, skip, st, p->mden));
   if (dbg_v) HELM_CK(cudaMemcpyAsync(dbg_v, fv, 2 * nx * cb, cudaMemcpyDeviceToDevice, st));
   // a3: Step 2
-  HELM_PK("apply_cbb", launch_apply_cbb(prec, fv, nullptr, fc, nx, p->h[0], p->h[1], p->wc[0], p->wc[1], p->omega * p->omega, ax.g,
-                                        ax.ginv, skip, st, p->mden));
   if (p->tabA && prec == kPrecF64)
-    HELM_CK(launch_tri2d_tab(2, nullptr, fc, p->tabA, p->rec, nullptr, p->partial, a, skip, st, p->prof.on ? &p->prof : nullptr));
+    HELM_CK(launch_tri2d_tab(2, nullptr, fc, p->tabA, p->rec, nullptr, p->partial, a, skip, st, p->prof.on ? &p->prof : nullptr,
+                             p->constA));
   else if (p->tabA)
     HELM_CK(launch_tri2d_t32(2, nullptr, fc, p->tabA, p->rec, nullptr, p->partial, a, skip, st, p->prof.on ? &p->prof : nullptr,
                              p->constA, p->dev_err));
   else
     HELM_CK(launch_tri2d(prec, 2, nullptr, fc, p->ustartA, p->rec, nullptr, p->partial, a, skip, st, p->prof.on ? &p->prof : nullptr, p->constA));
-  HELM_PK("reduce_faces", launch_reduce_faces(prec, p->partial, fw, nx, nparts, one, one, skip, st));
+  HELM_PK("faces_cbb", launch_faces_cbb(prec, p->partial, nparts, one, one, fw, fv, fc, nx, p->h[0], p->h[1], p->wc[0],
+                                        p->wc[1], p->omega * p->omega, ax.g, ax.ginv, skip, st, p->mden));
   if (dbg_w) HELM_CK(cudaMemcpyAsync(dbg_w, fw, 2 * nx * cb, cudaMemcpyDeviceToDevice, st));
   // a4: Step 3
-  HELM_PK("apply_cbb", launch_apply_cbb(prec, fv, fw, fc, nx, p->h[0], p->h[1], p->wc[0], p->wc[1], p->omega * p->omega, ax.g,
-                                        ax.ginv, skip, st, p->mden));
   if (p->tabB && prec == kPrecF64)
-    HELM_CK(launch_tri2d_tab(3, p->fhat, fc, p->tabB, p->rec, p->dbuf, nullptr, a, skip, st, p->prof.on ? &p->prof : nullptr));
+    HELM_CK(launch_tri2d_tab(3, p->fhat, fc, p->tabB, p->rec, p->dbuf, nullptr, a, skip, st, p->prof.on ? &p->prof : nullptr,
+                             p->constB));
   else if (p->tabB)
     HELM_CK(launch_tri2d_t32(3, p->fhat, fc, p->tabB, p->rec, p->dbuf, nullptr, a, skip, st, p->prof.on ? &p->prof : nullptr,
                              p->constB, p->dev_err));

@@ -54,7 +54,15 @@ size_t line_tables_bytes(int64_t nx, int64_t n1, int64_t nchunks);
 cudaError_t launch_line_tables(void* tables, const Solve2DArgs& a, int step, cudaStream_t st);
 cudaError_t launch_tri2d_tab(int step, const void* fhat, const void* faces, const void* tables, void* rec,
                              void* out, void* partial, const Solve2DArgs& a, const int* skip, cudaStream_t st,
-                             Profiler* prof);
+                             Profiler* prof, const void* consts);
+// Lines per block of its two passes, and so of one face partial (steps 1, 2).
+// A block's FP64 work is tens of us long at 128 lines on one SM, so lines are
+// spread over more SMs until every SM has 128-line blocks to share: at 129^2
+// pass 2 takes 17 us with 128 lines and 14 with 32 (launch and timing 5 of it).
+// Beyond that 128 lines write a quarter of the partials.
+inline int tri2d_tab_lines(int64_t n1, int64_t nchunks) {
+  return (n1 + 127) / 128 * nchunks < 8 * 152 ? 32 : 128;
+}
 // complex64 path with a per-plan pivot table (1/u_j rounded from FP64, chunk
 // constants): table memory per line type, building it, and the step launch.
 size_t line_tables32_bytes(int64_t nx, int64_t n1, int64_t nchunks);
@@ -64,14 +72,14 @@ cudaError_t launch_tri2d_t32(int step, const void* fhat, const void* faces, cons
                              void* partial, const Solve2DArgs& a, const int* skip, cudaStream_t st, Profiler* prof,
                              const void* consts, int* err);
 size_t chunk_record_bytes(int prec);
-// out[face][ix] = scale_face * sum_w partial (complex scales, face 0 then 1).
-cudaError_t launch_reduce_faces(int prec, const void* partial, void* out, int64_t nx, int64_t nwarps,
-                                const double* scale0, const double* scale1, const int* skip, cudaStream_t st);
-// C_bb of the auxiliary with wrap factor g (eq. Cbb; g = 1: periodic).
+// Boundary faces from the partials, v[face][ix] = s_face * sum partial (complex
+// scales, face 0 then 1), then out = C_bb (v + prev) (prev may be null): C_bb
+// of the auxiliary with wrap factor g (eq. Cbb; g = 1: periodic).
 // wx, wy: w of the absorbing x ends and x1 faces (0 on a Neumann axis).
-cudaError_t launch_apply_cbb(int prec, const void* in, const void* in2, void* out, int64_t nx, double hx,
-                             double h1, double wx, double wy, double p, const double* g, const double* ginv,
-                             const int* skip, cudaStream_t st, double mden);
+cudaError_t launch_faces_cbb(int prec, const void* partial, int64_t nparts, const double* s0, const double* s1,
+                             void* v, const void* prev, void* out, int64_t nx, double hx, double h1, double wx,
+                             double wy, double p, const double* g, const double* ginv, const int* skip,
+                             cudaStream_t st, double mden);
 
 // Refinement state kept on the device (one per plan).
 struct RefineState {

@@ -235,15 +235,28 @@ __global__ void __launch_bounds__(128) k_tri_pass1(const typename cpx<T>::type* 
 //
 // Each chunk's carry step is an affine map: Y(k) = a_k + pe_k Y(k-1) forward,
 // X(k) = c_k + q_k X(k+1) backward with c_k = bsum_k + cc_k Y(k-1) and
-// q_k = -b we_k (stored in rec.we).  A block takes kCarryLines lines (one per
+// q_k = -b we_k (stored in rec.we).  A block takes carry_lines() lines (one per
 // x thread, so every load of a field is a contiguous run of lines) and splits
-// their chunks into kCarrySeg contiguous segments (one per y thread).  Each
-// thread composes the maps of its segment, the segment maps are folded in
-// shared memory to give each segment its incoming carry, and each thread then
-// runs its segment's recurrence from that carry.  Same recurrences as the
-// sequential scan, regrouped once, in the precision of the records.
-constexpr int kCarryLines = 16;
+// their chunks into blockDim.y contiguous segments (one per y thread).  Each
+// thread composes the maps of its segment, one thread per line folds the
+// segment maps in shared memory into each segment's incoming carry, and each
+// thread then runs its segment's recurrence from that carry.  Same recurrences
+// as the sequential scan, regrouped once, in the precision of the records.
+//
+// Bound, complex128: the FP64 pipe (2 fused multiply-adds per clock and SM, so
+// one instruction of a warp takes 16 clocks however few of its lanes work).
+// The fold is therefore done once per line by half a warp (a chain of <= 31
+// steps of 4 fused operations) and not by every segment for itself, which
+// took 16 warps x 15 steps on average: at 129^2 that was most of 39 us, now
+// 16 (with the timing's own 4-5); at 8192 x 4096 418 us, now 283.  Segments hold at least
+// kCarryMinSeg chunks, so that short lines neither fold nor launch empty ones.
+// 128 bytes of lines, so that every load of a field is whole lines of memory
+template <typename T>
+__host__ __device__ constexpr int carry_lines() {
+  return 64 / (int)sizeof(T);
+}
 constexpr int kCarrySeg = 32;
+constexpr int kCarryMinSeg = 4;
 // chunk records loaded ahead of each recurrence; complex64 takes half as many
 // so that two blocks fit on an SM (every block of a 4096-line solve resident)
 template <typename T>
@@ -251,17 +264,42 @@ __host__ __device__ constexpr int carry_batch() {
   return sizeof(T) == 4 ? 4 : 8;
 }
 
+// Carry entering each segment from the segments' maps (c, p) of one line:
+// shC[g] <- carry into segment g; dir +1 from the first segment, -1 from the
+// last.  The loads of kB segments are issued before their chain.
+template <typename C, int NL>
+__device__ __forceinline__ void carry_fold(C (*shC)[NL], const C (*shP)[NL], int lx, int nseg, int dir) {
+  constexpr int kB = 8;
+  C v = mk<C>(0, 0);
+  const int g0 = dir > 0 ? 0 : nseg - 1;
+  for (int b = 0; b < nseg; b += kB) {
+    C c[kB], p[kB];
+#pragma unroll
+    for (int t = 0; t < kB; ++t)
+      if (b + t < nseg) {
+        c[t] = shC[g0 + dir * (b + t)][lx];
+        p[t] = shP[g0 + dir * (b + t)][lx];
+      }
+#pragma unroll
+    for (int t = 0; t < kB; ++t)
+      if (b + t < nseg) {
+        shC[g0 + dir * (b + t)][lx] = v;
+        v = cfma(p[t], v, c[t]);
+      }
+  }
+}
+
 template <typename T>
-__global__ void __launch_bounds__(kCarryLines* kCarrySeg, sizeof(T) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(carry_lines<T>() * kCarrySeg, 2)
     k_tri_carry(RecSoA<typename cpx<T>::type> rec, int64_t n1, int64_t K, const int* __restrict__ skip) {
   using C = typename cpx<T>::type;
-  constexpr int B = carry_batch<T>();
+  constexpr int B = carry_batch<T>(), NL = carry_lines<T>();
   if (skip && *skip) return;  // uniform over the grid
-  __shared__ C shC[kCarrySeg][kCarryLines], shP[kCarrySeg][kCarryLines];
-  const int lx = threadIdx.x, sg = threadIdx.y;
-  const int64_t l = (int64_t)blockIdx.x * kCarryLines + lx;
+  __shared__ C shC[kCarrySeg][NL], shP[kCarrySeg][NL];
+  const int lx = threadIdx.x, sg = threadIdx.y, nseg = blockDim.y;
+  const int64_t l = (int64_t)blockIdx.x * NL + lx;
   const bool act = l < n1;
-  const int64_t S = (K + kCarrySeg - 1) / kCarrySeg;
+  const int64_t S = (K + nseg - 1) / nseg;
   const int64_t k0 = min(K, sg * S), k1 = min(K, k0 + S);
   const C one = mk<C>(1, 0), zero = mk<C>(0, 0);
   // forward: compose the segment's maps
@@ -279,15 +317,16 @@ __global__ void __launch_bounds__(kCarryLines* kCarrySeg, sizeof(T) == 4 ? 2 : 1
       for (int t = 0; t < B; ++t)
         if (kb + t < k1) {
           const C pk = pv[t];
-          A = cadd(av[t], cmul(pk, A));
+          A = cfma(pk, A, av[t]);
           P = cmul(pk, P);
         }
     }
   shC[sg][lx] = A;
   shP[sg][lx] = P;
   __syncthreads();
-  C Y = zero;
-  for (int g = 0; g < sg; ++g) Y = cadd(shC[g][lx], cmul(shP[g][lx], Y));
+  if (sg == 0) carry_fold<C, NL>(shC, shP, lx, nseg, 1);
+  __syncthreads();
+  C Y = shC[sg][lx];
   // forward recurrence; c_k replaces bsum_k
   if (act)
     for (int64_t kb = k0; kb < k1; kb += B) {
@@ -306,12 +345,12 @@ __global__ void __launch_bounds__(kCarryLines* kCarrySeg, sizeof(T) == 4 ? 2 : 1
         if (kb + t < k1) {
           const int64_t i = (kb + t) * n1 + l;
           rec.a[i] = Y;  // Y(k-1)
-          rec.bsum[i] = cadd(bv[t], cmul(cv[t], Y));
-          Y = cadd(av[t], cmul(pv[t], Y));
+          rec.bsum[i] = cfma(cv[t], Y, bv[t]);
+          Y = cfma(pv[t], Y, av[t]);
         }
     }
-  __syncthreads();
-  // backward: compose the segment's maps, last chunk first
+  // backward: compose the segment's maps, last chunk first (each thread reads
+  // the c_k it wrote)
   C Cs = zero, Q = one;
   if (act)
     for (int64_t kb = k1 - 1; kb >= k0; kb -= B) {
@@ -326,15 +365,17 @@ __global__ void __launch_bounds__(kCarryLines* kCarrySeg, sizeof(T) == 4 ? 2 : 1
       for (int t = 0; t < B; ++t)
         if (kb - t >= k0) {
           const C qk = qv[t];
-          Cs = cadd(cv[t], cmul(qk, Cs));
+          Cs = cfma(qk, Cs, cv[t]);
           Q = cmul(qk, Q);
         }
     }
+  __syncthreads();  // every thread has its Y
   shC[sg][lx] = Cs;
   shP[sg][lx] = Q;
   __syncthreads();
-  C X = zero;
-  for (int g = kCarrySeg - 1; g > sg; --g) X = cadd(shC[g][lx], cmul(shP[g][lx], X));
+  if (sg == 0) carry_fold<C, NL>(shC, shP, lx, nseg, -1);
+  __syncthreads();
+  C X = shC[sg][lx];
   if (act)
     for (int64_t kb = k1 - 1; kb >= k0; kb -= B) {
       C cv[B], qv[B];
@@ -348,29 +389,41 @@ __global__ void __launch_bounds__(kCarryLines* kCarrySeg, sizeof(T) == 4 ? 2 : 1
       for (int t = 0; t < B; ++t)
         if (kb - t >= k0) {
           rec.bsum[(kb - t) * n1 + l] = X;  // X(k+1)
-          X = cadd(cv[t], cmul(qv[t], X));
+          X = cfma(qv[t], X, cv[t]);
         }
     }
 }
 
-// Sum the face contributions of a block's 128 lines for each of its `cnt`
+// Threads of the carry scan: a block's lines by the segments of K chunks.
+template <typename T>
+inline dim3 carry_block(int64_t K) {
+  const int64_t seg = std::min<int64_t>(kCarrySeg, (K + kCarryMinSeg - 1) / kCarryMinSeg);
+  return dim3(carry_lines<T>(), (unsigned)std::max<int64_t>(1, seg));
+}
+template <typename T>
+inline unsigned carry_grid(int64_t n1) {
+  return (unsigned)((n1 + carry_lines<T>() - 1) / carry_lines<T>());
+}
+
+// Sum the face contributions of a block's BS lines for each of its `cnt`
 // rows (red[face][row][thread]) and write one partial per block and row:
 // partial[(face * nparts + blk) * nx + row0 + t].  Fixed summation order.
-template <typename C, int CH>
+template <typename C, int CH, int BS = 128>
 __device__ __forceinline__ void block_face_sums(C* red, int cnt, C* __restrict__ partial, int64_t blk,
                                                 int64_t nparts, int64_t nx, int64_t row0) {
   constexpr int NQ = 2 * CH;    // sums: face * CH + row
   constexpr int SP = NQ + 1;    // padded stride of the segment sums
-  __shared__ C seg[16 * SP];
+  constexpr int NG = BS / 8;    // segments of 8 lines
+  __shared__ C seg[NG * SP];
   __syncthreads();
-  // stage 1: thread -> (sum q, segment g of 8 consecutive lines, lines g, g+16,
-  // ..., g+112); a half-warp reads 16 consecutive values (no bank conflicts)
-  for (int w = threadIdx.x; w < NQ * 16; w += blockDim.x) {
-    const int q = w >> 4, g = w & 15;
-    const C* src = red + q * 128 + g;
+  // stage 1: thread -> (sum q, segment g of the 8 lines g, g+NG, ...); BS =
+  // 128: a half-warp reads 16 consecutive values (no bank conflicts)
+  for (int w = threadIdx.x; w < NQ * NG; w += blockDim.x) {
+    const int q = w / NG, g = w % NG;
+    const C* src = red + q * BS + g;
     C acc = src[0];
 #pragma unroll
-    for (int i = 1; i < 8; ++i) acc = cadd(acc, src[16 * i]);
+    for (int i = 1; i < 8; ++i) acc = cadd(acc, src[NG * i]);
     seg[g * SP + q] = acc;
   }
   __syncthreads();
@@ -379,7 +432,7 @@ __device__ __forceinline__ void block_face_sums(C* red, int cnt, C* __restrict__
     if (t >= cnt) continue;
     C acc = seg[q];
 #pragma unroll
-    for (int g = 1; g < 16; ++g) acc = cadd(acc, seg[g * SP + q]);
+    for (int g = 1; g < NG; ++g) acc = cadd(acc, seg[g * SP + q]);
     partial[(face * nparts + blk) * nx + row0 + t] = acc;
   }
 }
@@ -538,6 +591,7 @@ template <int STEP, int CH>
 __global__ void __launch_bounds__(128) k_tri_pass1_tab(const double2* __restrict__ fhat,
                                                        const double2* __restrict__ faces, LineTables tb,
                                                        RecSoA<double2> rec, Solve2DArgs a,
+                                                       const void* __restrict__ consts,
                                                        const int* __restrict__ skip) {
   using C = double2;
   if (skip && *skip) return;
@@ -547,9 +601,10 @@ __global__ void __launch_bounds__(128) k_tri_pass1_tab(const double2* __restrict
   const int64_t k = blockIdx.y;
   const int64_t s = k * CH, e = min(s + (int64_t)CH, nx) - 1;
   const int cnt = (int)(e - s + 1);
-  const C scal = (STEP == 2) ? mk<C>(1, 0) : mk<C>(a.invmu[2 * l], a.invmu[2 * l + 1]);
-  const C wl = step3_weight<C>(a, l);
-  const double par = a.parA[l];
+  const LineConst<C> lt = line_const<C>(consts, n1);
+  const C scal = lt.scal[l];
+  const C wl = lt.wl[l];
+  const double par = lt.par[l].x;
   const C* f1 = faces;
   const C* fn = faces + nx;
   C rr[CH], mj[CH], wj[CH];
@@ -565,18 +620,19 @@ __global__ void __launch_bounds__(128) k_tri_pass1_tab(const double2* __restrict
 #pragma unroll
   for (int t = 0; t < CH; ++t) {
     if (t >= cnt) break;
-    ylo = (t == 0) ? rr[t] : csub(rr[t], cmul(mj[t], ylo));
-    bsum = cadd(bsum, cmul(wj[t], ylo));
+    ylo = (t == 0) ? rr[t] : cfms(rr[t], mj[t], ylo);
+    bsum = cfma(wj[t], ylo, bsum);
   }
   rec.a[k * n1 + l] = ylo;
   rec.bsum[k * n1 + l] = bsum;
 }
 
-template <int STEP, int CH>
-__global__ void __launch_bounds__(128) k_tri_pass2_tab(const double2* __restrict__ fhat,
+template <int STEP, int CH, int BS>
+__global__ void __launch_bounds__(BS) k_tri_pass2_tab(const double2* __restrict__ fhat,
                                                        const double2* __restrict__ faces, LineTables tb,
                                                        RecSoA<double2> rec, double2* __restrict__ out,
                                                        double2* __restrict__ partial, Solve2DArgs a,
+                                                       const void* __restrict__ consts,
                                                        const int* __restrict__ skip) {
   using C = double2;
   if (skip && *skip) return;
@@ -588,13 +644,13 @@ __global__ void __launch_bounds__(128) k_tri_pass2_tab(const double2* __restrict
   const int64_t k = blockIdx.y;
   const int64_t s = k * CH, e = min(s + (int64_t)CH, nx) - 1;
   const int cnt = (int)(e - s + 1);
-  const LineParams lp = line_params(STEP, a, lc);
-  const LineCoef<C> co = line_coef<C>(lp.sre, lp.sim, a.hx, a.wx, a.mden);
-  const C scal = (STEP == 2) ? mk<C>(1, 0) : mk<C>(a.invmu[2 * lc], a.invmu[2 * lc + 1]);
-  const C twl = mk<C>(a.tw[2 * lc], a.tw[2 * lc + 1]);
-  const C wl = step3_weight<C>(a, lc);
-  const double par = a.parA[lc];
-  const C sig = mk<C>(a.sigA[2 * lc], a.sigA[2 * lc + 1]);
+  const LineConst<C> lt = line_const<C>(consts, n1);
+  const C b = lt.b[lc];
+  const C scal = lt.scal[lc];
+  const C twl = lt.twl[lc];
+  const C wl = lt.wl[lc];
+  const double par = lt.par[lc].x;
+  const C sig = lt.sig[lc];
   const C* f1 = faces;
   const C* fn = faces + nx;
   const C zero = mk<C>(0, 0);
@@ -611,19 +667,19 @@ __global__ void __launch_bounds__(128) k_tri_pass2_tab(const double2* __restrict
 #pragma unroll
   for (int t = 0; t < CH; ++t) {
     if (t < cnt) {
-      yp = csub(y[t], cmul(mj[t], yp));
+      yp = cfms(y[t], mj[t], yp);
       y[t] = yp;
     }
   }
-  // face contributions of the block's 128 lines, reduced per row in shared memory
-  __shared__ C red[2 * CH * 128];
-  const int64_t nparts = (n1 + 127) / 128;
+  // face contributions of the block's BS lines, reduced per row in shared memory
+  __shared__ C red[2 * CH * BS];
+  const int64_t nparts = (n1 + BS - 1) / BS;
   C xn = rec.bsum[k * n1 + lc];  // X(k+1)
 #pragma unroll
   for (int t = CH - 1; t >= 0; --t) {
     if (t < cnt) {
       const int64_t j = s + t;
-      const C x = cmul(csub(y[t], cmul(co.b, xn)), iu[t]);
+      const C x = cmul(cfms(y[t], b, xn), iu[t]);
       xn = x;
       if (STEP == 3) {
         if (act) out[j * n1 + lc] = x;
@@ -637,12 +693,12 @@ __global__ void __launch_bounds__(128) k_tri_pass2_tab(const double2* __restrict
           s1 = tt;
           sn = cscale(tt, par);
         }
-        red[(0 * CH + t) * 128 + threadIdx.x] = s1;
-        red[(1 * CH + t) * 128 + threadIdx.x] = sn;
+        red[(0 * CH + t) * BS + threadIdx.x] = s1;
+        red[(1 * CH + t) * BS + threadIdx.x] = sn;
       }
     }
   }
-  if (STEP != 3) block_face_sums<C, CH>(red, cnt, partial, (int64_t)blockIdx.x, nparts, nx, s);
+  if (STEP != 3) block_face_sums<C, CH, BS>(red, cnt, partial, (int64_t)blockIdx.x, nparts, nx, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -1110,40 +1166,11 @@ __global__ void k_pivots(typename cpx<T>::type* __restrict__ ustart, Solve2DArgs
   }
 }
 
-// Sum the per-block partials: out[face * nx + ix] = scale * sum_w partial.
-// Four lanes per output (lanes j, j+8, j+16, j+24 of a warp), each summing
-// the partials w = q, q+4, ... (independent loads), combined by two fixed
-// shuffles: a fixed summation order.
-constexpr int kFaceLanes = 4;
-template <typename T>
-__global__ void __launch_bounds__(256) k_reduce_faces(const typename cpx<T>::type* __restrict__ partial,
-                                                      typename cpx<T>::type* __restrict__ out, int64_t nx,
-                                                      int64_t nwarps, double s0r, double s0i, double s1r,
-                                                      double s1i, const int* __restrict__ skip) {
-  using C = typename cpx<T>::type;
-  if (skip && *skip) return;
-  const int lane = threadIdx.x & 31, q = lane >> 3;
-  const int64_t i = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) / kFaceLanes + (lane & 7);
-  const bool act = i < 2 * nx;
-  const int64_t face = act ? i / nx : 0, ix = act ? i - face * nx : 0;
-  C acc = mk<C>(0, 0);
-  if (act) {
-    const C* src = partial + (face * nwarps) * nx + ix;
-#pragma unroll 8
-    for (int64_t w = q; w < nwarps; w += kFaceLanes) acc = cadd(acc, src[w * nx]);
-  }
-  for (int off = 8; off < 32; off <<= 1) {
-    acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
-    acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
-  }
-  if (act && q == 0) out[i] = cmul(acc, face == 0 ? mk<C>(s0r, s0i) : mk<C>(s1r, s1i));
-}
-
 // C_bb applied to the x1 faces (eqs. BminA, Cbb):
 //   c_1 = D11 M v_1 + E11 K v_1 + D1n M v_n + E1n K v_n,  c_n symmetric,
 // with D11 = (1 + i w h1)/h1 - p h1/3, D1n = -1/h1 - p h1/6, E11 = h1/3,
 // E1n = h1/6 (p = w^2 for the outer problem), M, K along x (spacing hx,
-// absorbing corners).  in = v (+ w if `in2`), out = c.
+// absorbing corners).
 struct CbbConsts {
   double md_end, md_in, mo;        // M rows: diagonal (end, inner), off-diagonal
   double kd_end_re, kd_end_im;     // K diagonal at the absorbing ends
@@ -1153,44 +1180,62 @@ struct CbbConsts {
   double gr, gi, gir, gii;         // g and 1/g: wrap entries of the gamma-circulant
 };
 
+// Boundary faces and C_bb in one launch: v[face][ix] = scale_face * sum_w
+// partial (written out), then out = C_bb (v + prev) with prev optional.
+//
+// A block takes kFaceRows rows and one halo row on either side (the rows of
+// C_bb along x), one lane per row; its eight warps are (face, q) with q = 0..3
+// summing the partials w = q, q+4, ... (independent loads), combined as
+// (q0 + q1) + (q2 + q3): a fixed summation order.  Bound: the launch and two
+// dependent loads at small sizes, the read of the partials (32/30 of it for
+// the halo) at large ones.  As two kernels, 2 x (6.6 + 8.7) us of a 129^2
+// complex128 solve; one of 8.1.
+constexpr int kFaceLanes = 4;
+constexpr int kFaceRows = 30;
 template <typename T>
-__global__ void k_apply_cbb(const typename cpx<T>::type* __restrict__ in,
-                            const typename cpx<T>::type* __restrict__ in2,
-                            typename cpx<T>::type* __restrict__ out, int64_t nx, CbbConsts k,
-                            const int* __restrict__ skip) {
+__global__ void __launch_bounds__(64 * kFaceLanes) k_faces_cbb(
+    const typename cpx<T>::type* __restrict__ partial, typename cpx<T>::type* __restrict__ v,
+    const typename cpx<T>::type* __restrict__ prev, typename cpx<T>::type* __restrict__ out, int64_t nx,
+    int64_t nparts, double s0r, double s0i, double s1r, double s1i, CbbConsts k, const int* __restrict__ skip) {
   using C = typename cpx<T>::type;
   using R = decltype(C().x);
-  if (skip && *skip) return;
-  const int64_t ix = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (ix >= nx) return;
-  auto get = [&](int face, int64_t j) -> C {
-    C v = in[face * nx + j];
-    if (in2) v = cadd(v, in2[face * nx + j]);
-    return v;
-  };
-  // M and K rows of x at ix
+  if (skip && *skip) return;  // uniform over the grid
+  __shared__ C red[kFaceLanes][2][32], val[2][32];
+  const int lane = threadIdx.x & 31, face = (threadIdx.x >> 5) & 1, q = threadIdx.x >> 6;
+  const int64_t ix = (int64_t)blockIdx.x * kFaceRows + lane - 1;
+  const bool act = ix >= 0 && ix < nx;
+  const bool mine = act && lane >= 1 && lane <= kFaceRows;  // a row of this block
+  const C zero = mk<C>(0, 0);
+  C acc = zero;
+  if (act) {
+    const C* src = partial + (face * nparts) * nx + ix;
+#pragma unroll 8
+    for (int64_t w = q; w < nparts; w += kFaceLanes) acc = cadd(acc, src[w * nx]);
+  }
+  red[q][face][lane] = acc;
+  __syncthreads();
+  if (q != 0) return;  // two warps go on, one per face
+  acc = cadd(cadd(acc, red[1][face][lane]), cadd(red[2][face][lane], red[3][face][lane]));
+  C x = cmul(acc, face == 0 ? mk<C>(s0r, s0i) : mk<C>(s1r, s1i));
+  if (mine) v[face * nx + ix] = x;
+  if (prev && act) x = cadd(prev[face * nx + ix], x);
+  // rows ix of M and K along x, of this face (zero beyond the ends: acc = 0)
+  const C lo = mk<C>(__shfl_up_sync(0xffffffffu, x.x, 1), __shfl_up_sync(0xffffffffu, x.y, 1));
+  const C hi = mk<C>(__shfl_down_sync(0xffffffffu, x.x, 1), __shfl_down_sync(0xffffffffu, x.y, 1));
   const bool end = (ix == 0 || ix == nx - 1);
   const R md = (R)(end ? k.md_end : k.md_in), mo = (R)k.mo, ko = (R)k.ko;
   const C kd = end ? mk<C>(k.kd_end_re, k.kd_end_im) : mk<C>(k.kd_in, 0.0);
-  C Mv[2], Kv[2];
-  for (int f = 0; f < 2; ++f) {
-    C v0 = get(f, ix);
-    C vm = ix > 0 ? get(f, ix - 1) : mk<C>(0, 0);
-    C vp = ix < nx - 1 ? get(f, ix + 1) : mk<C>(0, 0);
-    C nb = cadd(vm, vp);
-    Mv[f] = cadd(cscale(v0, md), cscale(nb, mo));
-    Kv[f] = cadd(cmul(v0, kd), cscale(nb, ko));
-  }
-  const C D11 = mk<C>(k.d11_re, k.d11_im);
-  const C D1n = mk<C>(k.d1n_re, 0.0);
-  const R E11 = (R)k.e11, E1n = (R)k.e1n;
-  // wrap entries of the gamma-circulant: first row x 1/g, last row x g
-  C c1 = cadd(cadd(cmul(D11, Mv[0]), cscale(Kv[0], E11)),
-              cmul(mk<C>(k.gir, k.gii), cadd(cmul(D1n, Mv[1]), cscale(Kv[1], E1n))));
-  C cn = cadd(cmul(mk<C>(k.gr, k.gi), cadd(cmul(D1n, Mv[0]), cscale(Kv[0], E1n))),
-              cadd(cmul(D11, Mv[1]), cscale(Kv[1], E11)));
-  out[ix] = c1;
-  out[nx + ix] = cn;
+  const C nb = cadd(lo, hi);
+  const C Mv = cadd(cscale(x, md), cscale(nb, mo));
+  const C Kv = cadd(cmul(x, kd), cscale(nb, ko));
+  // own part of this face's row, and this face's part of the other face's row
+  // (wrap entries of the gamma-circulant: first row x 1/g, last row x g)
+  const C own = cadd(cmul(mk<C>(k.d11_re, k.d11_im), Mv), cscale(Kv, (R)k.e11));
+  const C cross = cmul(face == 0 ? mk<C>(k.gr, k.gi) : mk<C>(k.gir, k.gii),
+                       cadd(cscale(Mv, (R)k.d1n_re), cscale(Kv, (R)k.e1n)));
+  val[face ^ 1][lane] = cross;
+  asm volatile("bar.sync 1, 64;" ::: "memory");  // the two remaining warps
+  if (mine) out[face * nx + ix] = cadd(own, val[face][lane]);
 }
 
 }  // namespace
@@ -1203,8 +1248,6 @@ cudaError_t launch_tri2d(int prec, int step, const void* fhat, const void* faces
   static const char* n2s[3] = {"tri_step1_pass2", "tri_step2_pass2", "tri_step3_pass2"};
   const int bs = 128;
   const dim3 grid((unsigned)((a.n1 + bs - 1) / bs), (unsigned)a.nchunks);
-  const unsigned gcar = (unsigned)((a.n1 + kCarryLines - 1) / kCarryLines);
-  const dim3 bcar(kCarryLines, kCarrySeg);
   const size_t nrec = (size_t)a.nchunks * a.n1;
 #define HELM_TRI(T, S, CH)                                                                                        \
   do {                                                                                                         \
@@ -1216,7 +1259,7 @@ cudaError_t launch_tri2d(int prec, int step, const void* fhat, const void* faces
     }                                                                                                          \
     {                                                                                                          \
       ProfScope ps(prof, ncs[S - 1], st);                                                                      \
-      k_tri_carry<T><<<gcar, bcar, 0, st>>>(rec_soa<C>(rec, nrec), a.n1, a.nchunks, skip);                         \
+      k_tri_carry<T><<<carry_grid<T>(a.n1), carry_block<T>(a.nchunks), 0, st>>>(rec_soa<C>(rec, nrec), a.n1, a.nchunks, skip);                         \
     }                                                                                                          \
     {                                                                                                          \
       ProfScope ps(prof, n2s[S - 1], st);                                                                      \
@@ -1241,15 +1284,13 @@ cudaError_t launch_tri2d(int prec, int step, const void* fhat, const void* faces
 
 cudaError_t launch_tri2d_tab(int step, const void* fhat, const void* faces, const void* tables, void* rec,
                              void* out, void* partial, const Solve2DArgs& a, const int* skip, cudaStream_t st,
-                             Profiler* prof) {
+                             Profiler* prof, const void* consts) {
   static const char* n1s[3] = {"tri_step1_pass1", "tri_step2_pass1", "tri_step3_pass1"};
   static const char* ncs[3] = {"tri_step1_carry", "tri_step2_carry", "tri_step3_carry"};
   static const char* n2s[3] = {"tri_step1_pass2", "tri_step2_pass2", "tri_step3_pass2"};
   if (a.ch != kChunkF64) return cudaErrorInvalidValue;
-  const int bs = 128;
+  const int bs = tri2d_tab_lines(a.n1, a.nchunks);
   const dim3 grid((unsigned)((a.n1 + bs - 1) / bs), (unsigned)a.nchunks);
-  const unsigned gcar = (unsigned)((a.n1 + kCarryLines - 1) / kCarryLines);
-  const dim3 bcar(kCarryLines, kCarrySeg);
   const size_t nrec = (size_t)a.nchunks * a.n1;
   const LineTables tb = line_tables(const_cast<void*>(tables), (size_t)a.nx * a.n1, nrec);
   RecSoA<double2> r = rec_soa<double2>(rec, nrec);
@@ -1261,16 +1302,20 @@ cudaError_t launch_tri2d_tab(int step, const void* fhat, const void* faces, cons
     {                                                                                                    \
       ProfScope ps(prof, n1s[S - 1], st);                                                                \
       k_tri_pass1_tab<S, kChunkF64><<<grid, bs, 0, st>>>((const double2*)fhat, (const double2*)faces, tb, r, \
-                                                         a, skip);                                     \
+                                                         a, consts, skip);                             \
     }                                                                                                    \
     {                                                                                                    \
       ProfScope ps(prof, ncs[S - 1], st);                                                                \
-      k_tri_carry<double><<<gcar, bcar, 0, st>>>(r, a.n1, a.nchunks, skip);                                 \
+      k_tri_carry<double><<<carry_grid<double>(a.n1), carry_block<double>(a.nchunks), 0, st>>>(r, a.n1, a.nchunks, skip);                                 \
     }                                                                                                    \
     {                                                                                                    \
       ProfScope ps(prof, n2s[S - 1], st);                                                                \
-      k_tri_pass2_tab<S, kChunkF64><<<grid, bs, 0, st>>>((const double2*)fhat, (const double2*)faces, tb, r, \
-                                                         (double2*)out, (double2*)partial, a, skip);   \
+      if (bs == 32)                                                                                     \
+        k_tri_pass2_tab<S, kChunkF64, 32><<<grid, bs, 0, st>>>(                                         \
+            (const double2*)fhat, (const double2*)faces, tb, r, (double2*)out, (double2*)partial, a, consts, skip); \
+      else                                                                                              \
+        k_tri_pass2_tab<S, kChunkF64, 128><<<grid, bs, 0, st>>>(                                        \
+            (const double2*)fhat, (const double2*)faces, tb, r, (double2*)out, (double2*)partial, a, consts, skip); \
     }                                                                                                    \
   } while (0)
   if (step == 1) HELM_TRI_TAB(1);
@@ -1289,8 +1334,6 @@ cudaError_t launch_tri2d_t32(int step, const void* fhat, const void* faces, cons
   if (a.ch != kChunkF32) return cudaErrorInvalidValue;
   const int bs = 128;
   const dim3 grid((unsigned)((a.n1 + bs - 1) / bs), (unsigned)a.nchunks);
-  const unsigned gcar = (unsigned)((a.n1 + kCarryLines - 1) / kCarryLines);
-  const dim3 bcar(kCarryLines, kCarrySeg);
   const size_t nrec = (size_t)a.nchunks * a.n1;
   const LineTables32 tb = line_tables32(const_cast<void*>(tables), (size_t)a.nx * a.n1, nrec, (size_t)a.n1);
   RecSoA<float2> r = rec_soa<float2>(rec, nrec);
@@ -1317,7 +1360,7 @@ cudaError_t launch_tri2d_t32(int step, const void* fhat, const void* faces, cons
       }                                                                                                       \
       {                                                                                                       \
         ProfScope ps(prof, ncs[S - 1], st);                                                                   \
-        k_tri_carry<float><<<gcar, bcar, 0, st>>>(r, a.n1, a.nchunks, skip);                                  \
+        k_tri_carry<float><<<carry_grid<float>(a.n1), carry_block<float>(a.nchunks), 0, st>>>(r, a.n1, a.nchunks, skip);                                  \
       }                                                                                                       \
       {                                                                                                       \
         ProfScope ps(prof, n2s[S - 1], st);                                                                   \
@@ -1333,7 +1376,7 @@ cudaError_t launch_tri2d_t32(int step, const void* fhat, const void* faces, cons
     }                                                                                                         \
     {                                                                                                         \
       ProfScope ps(prof, ncs[S - 1], st);                                                                     \
-      k_tri_carry<float><<<gcar, bcar, 0, st>>>(r, a.n1, a.nchunks, skip);                                    \
+      k_tri_carry<float><<<carry_grid<float>(a.n1), carry_block<float>(a.nchunks), 0, st>>>(r, a.n1, a.nchunks, skip);                                    \
     }                                                                                                         \
     {                                                                                                         \
       ProfScope ps(prof, n2s[S - 1], st);                                                                     \
@@ -1399,22 +1442,10 @@ cudaError_t launch_pivots(int prec, void* ustart, const Solve2DArgs& a, int step
 
 size_t chunk_record_bytes(int prec) { return prec == kPrecF64 ? sizeof(ChunkRec<double2>) : sizeof(ChunkRec<float2>); }
 
-cudaError_t launch_reduce_faces(int prec, const void* partial, void* out, int64_t nx, int64_t nwarps,
-                                const double* s0, const double* s1, const int* skip, cudaStream_t st) {
-  const int bs = 256;
-  const unsigned grid = (unsigned)((2 * nx * kFaceLanes + bs - 1) / bs);
-  if (prec == kPrecF64)
-    k_reduce_faces<double><<<grid, bs, 0, st>>>((const double2*)partial, (double2*)out, nx, nwarps, s0[0], s0[1],
-                                                s1[0], s1[1], skip);
-  else
-    k_reduce_faces<float><<<grid, bs, 0, st>>>((const float2*)partial, (float2*)out, nx, nwarps, s0[0], s0[1], s1[0],
-                                               s1[1], skip);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_apply_cbb(int prec, const void* in, const void* in2, void* out, int64_t nx, double hx,
-                             double h1, double wx, double wy, double p, const double* g, const double* ginv,
-                             const int* skip, cudaStream_t st, double mden) {
+cudaError_t launch_faces_cbb(int prec, const void* partial, int64_t nparts, const double* s0, const double* s1,
+                             void* v, const void* prev, void* out, int64_t nx, double hx, double h1, double wx,
+                             double wy, double p, const double* g, const double* ginv, const int* skip,
+                             cudaStream_t st, double mden) {
   // the entries of eqs. BminA, Cbb once, in double, on the host
   const MassCoef mx = mass_coef(hx, mden), m1 = mass_coef(h1, mden);
   CbbConsts k;
@@ -1434,12 +1465,14 @@ cudaError_t launch_apply_cbb(int prec, const void* in, const void* in2, void* ou
   k.gi = g[1];
   k.gir = ginv[0];
   k.gii = ginv[1];
-  const int bs = 256;
-  const unsigned grid = (unsigned)((nx + bs - 1) / bs);
+  const int bs = 64 * kFaceLanes;
+  const unsigned grid = (unsigned)((nx + kFaceRows - 1) / kFaceRows);
   if (prec == kPrecF64)
-    k_apply_cbb<double><<<grid, bs, 0, st>>>((const double2*)in, (const double2*)in2, (double2*)out, nx, k, skip);
+    k_faces_cbb<double><<<grid, bs, 0, st>>>((const double2*)partial, (double2*)v, (const double2*)prev,
+                                             (double2*)out, nx, nparts, s0[0], s0[1], s1[0], s1[1], k, skip);
   else
-    k_apply_cbb<float><<<grid, bs, 0, st>>>((const float2*)in, (const float2*)in2, (float2*)out, nx, k, skip);
+    k_faces_cbb<float><<<grid, bs, 0, st>>>((const float2*)partial, (float2*)v, (const float2*)prev, (float2*)out,
+                                            nx, nparts, s0[0], s0[1], s1[0], s1[1], k, skip);
   return cudaGetLastError();
 }
 
