@@ -214,9 +214,10 @@ int helm_set_precision_routing(helm_plan_t p, double tau);
  *                             1024 rows, 512 in complex128).
  *   HELM_VARIANT_INNER_TILES  3D: tiles of 16 inner modes per CTA (1..8;
  *                             default 1..4 by grid size).
- *   HELM_VARIANT_TRI2D        2D complex64: 0 = bulk-copy fed passes where
- *                             the x1 length is even (default), 1 = register-
- *                             tile passes.
+ *   HELM_VARIANT_TRI2D        2D complex64: 0 = one kernel per step on grids
+ *                             of up to 4 Mi unknowns and 2048 rows, beyond
+ *                             them bulk-copy fed passes where the x1 length
+ *                             is even (default), 1 = register-tile passes.
  *   HELM_VARIANT_DFT          complex64 plans whose contiguous transformed
  *                             axis (x1 in 2D, the inner axis in 3D) has at
  *                             most 128 nodes: 0 = FFT kernels (default), 1 =

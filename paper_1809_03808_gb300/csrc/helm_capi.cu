@@ -448,45 +448,35 @@ int solve2d_core(helm_plan* p, const void* in, int in_is_double, void* out, int 
   const void* sco = f64 ? (const void*)ax.sc_out : (const void*)ax.sc_out32;
   const double one[2] = {1.0, 0.0}, inv_n1[2] = {1.0 / (double)n1, 0.0};
   const double en_n1[2] = {ax.en[0] / (double)n1, ax.en[1] / (double)n1};
-  // face partials: one per block of lines of the step kernels
-  const int64_t lpb = p->tabB && f64 ? tri2d_tab_lines(n1, a.nchunks) : 128;
+  // kernels of the three steps, and face partials: one per block of their lines
+  const int fused = p->tabB && !p->tri_regs ? tri2d_fused_lines(prec, nx, n1, a.nchunks) : 0;
+  const int64_t lpb = fused ? fused : p->tabB && f64 ? tri2d_tab_lines(n1, a.nchunks) : 128;
   const int64_t nparts = (n1 + lpb - 1) / lpb;
+  Profiler* prof = p->prof.on ? &p->prof : nullptr;
+  auto step = [&](int which, const void* rhs, const void* face, void* x, void* part) -> cudaError_t {
+    const bool A = which == 2;
+    const void* tab = A ? p->tabA : p->tabB;
+    const void* cst = A ? p->constA : p->constB;
+    if (fused) return launch_tri2d_fused(prec, which, rhs, face, tab, x, part, a, skip, st, prof, cst);
+    if (tab && f64) return launch_tri2d_tab(which, rhs, face, tab, p->rec, x, part, a, skip, st, prof, cst);
+    if (tab) return launch_tri2d_t32(which, rhs, face, tab, p->rec, x, part, a, skip, st, prof, cst, p->dev_err);
+    return launch_tri2d(prec, which, rhs, face, A ? p->ustartA : p->ustartB, p->rec, x, part, a, skip, st, prof, cst);
+  };
   HELM_PK("dft_fwd", launch_dft_rows(prec, in, in_is_double, p->fhat, fhat_mode, nx, ax.dft, tw, -1, 1.0, 0.0, sci,
                                      nullptr, skip, st, p->dev_err));
   if (dbg_fhat) HELM_CK(cudaMemcpyAsync(dbg_fhat, p->fhat, nx * n1 * cb, cudaMemcpyDeviceToDevice, st));
   // a2: Step 1
-  if (p->tabB && prec == kPrecF64)
-    HELM_CK(launch_tri2d_tab(1, p->fhat, nullptr, p->tabB, p->rec, nullptr, p->partial, a, skip, st, p->prof.on ? &p->prof : nullptr,
-                             p->constB));
-  else if (p->tabB)
-    HELM_CK(launch_tri2d_t32(1, p->fhat, nullptr, p->tabB, p->rec, nullptr, p->partial, a, skip, st, p->prof.on ? &p->prof : nullptr,
-                             p->constB, p->dev_err));
-  else
-    HELM_CK(launch_tri2d(prec, 1, p->fhat, nullptr, p->ustartB, p->rec, nullptr, p->partial, a, skip, st, p->prof.on ? &p->prof : nullptr, p->constB));
+  HELM_CK(step(1, p->fhat, nullptr, nullptr, p->partial));
   HELM_PK("faces_cbb", launch_faces_cbb(prec, p->partial, nparts, inv_n1, en_n1, fv, nullptr, fc, nx, p->h[0], p->h[1],
                                         p->wc[0], p->wc[1], p->omega * p->omega, ax.g, ax.ginv, skip, st, p->mden));
   if (dbg_v) HELM_CK(cudaMemcpyAsync(dbg_v, fv, 2 * nx * cb, cudaMemcpyDeviceToDevice, st));
   // a3: Step 2
-  if (p->tabA && prec == kPrecF64)
-    HELM_CK(launch_tri2d_tab(2, nullptr, fc, p->tabA, p->rec, nullptr, p->partial, a, skip, st, p->prof.on ? &p->prof : nullptr,
-                             p->constA));
-  else if (p->tabA)
-    HELM_CK(launch_tri2d_t32(2, nullptr, fc, p->tabA, p->rec, nullptr, p->partial, a, skip, st, p->prof.on ? &p->prof : nullptr,
-                             p->constA, p->dev_err));
-  else
-    HELM_CK(launch_tri2d(prec, 2, nullptr, fc, p->ustartA, p->rec, nullptr, p->partial, a, skip, st, p->prof.on ? &p->prof : nullptr, p->constA));
+  HELM_CK(step(2, nullptr, fc, nullptr, p->partial));
   HELM_PK("faces_cbb", launch_faces_cbb(prec, p->partial, nparts, one, one, fw, fv, fc, nx, p->h[0], p->h[1], p->wc[0],
                                         p->wc[1], p->omega * p->omega, ax.g, ax.ginv, skip, st, p->mden));
   if (dbg_w) HELM_CK(cudaMemcpyAsync(dbg_w, fw, 2 * nx * cb, cudaMemcpyDeviceToDevice, st));
   // a4: Step 3
-  if (p->tabB && prec == kPrecF64)
-    HELM_CK(launch_tri2d_tab(3, p->fhat, fc, p->tabB, p->rec, p->dbuf, nullptr, a, skip, st, p->prof.on ? &p->prof : nullptr,
-                             p->constB));
-  else if (p->tabB)
-    HELM_CK(launch_tri2d_t32(3, p->fhat, fc, p->tabB, p->rec, p->dbuf, nullptr, a, skip, st, p->prof.on ? &p->prof : nullptr,
-                             p->constB, p->dev_err));
-  else
-    HELM_CK(launch_tri2d(prec, 3, p->fhat, fc, p->ustartB, p->rec, p->dbuf, nullptr, a, skip, st, p->prof.on ? &p->prof : nullptr, p->constB));
+  HELM_CK(step(3, p->fhat, fc, p->dbuf, nullptr));
   // a5: inverse DFT along x1 (eq. step3IFFTz3coeff)
   HELM_PK("dft_inv", launch_dft_rows(prec, p->dbuf, prec == kPrecF64, out, out_mode, nx, ax.dft, tw, +1, 1.0 / (double)n1,
                                      accum_scale, nullptr, sco, skip, st));
@@ -671,9 +661,11 @@ int alloc_buffers_2d(helm_plan* p) {
   const int64_t nx = p->n[0], n1 = p->n[1], N = nx * n1;
   const size_t cb = cbytes(p->prec);
   int rc;
-  p->nwarps = (n1 + 31) / 32;
   p->face_len = nx;
   const Solve2DArgs a = args2d(p);
+  // face partials: of the kernels with the fewest lines per block
+  const int fused = tri2d_fused_lines(p->prec, nx, n1, a.nchunks);
+  p->nwarps = (n1 + (fused ? fused : 32) - 1) / (fused ? fused : 32);
   const size_t nrec = (size_t)a.nchunks * n1;
   if ((rc = dev_alloc(p, &p->fhat, N * cb)) || (rc = dev_alloc(p, &p->dbuf, N * cb)) ||
       (rc = dev_alloc(p, &p->partial, 2 * p->nwarps * nx * cb)) || (rc = dev_alloc(p, &p->faces, 8 * nx * cb)) ||

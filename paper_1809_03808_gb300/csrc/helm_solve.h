@@ -71,6 +71,13 @@ cudaError_t launch_line_tables32(void* tables, const Solve2DArgs& a, int step, c
 cudaError_t launch_tri2d_t32(int step, const void* fhat, const void* faces, const void* tables, void* rec, void* out,
                              void* partial, const Solve2DArgs& a, const int* skip, cudaStream_t st, Profiler* prof,
                              const void* consts, int* err);
+// One step as one kernel, where a block holds whole lines: lines per block (and
+// per face partial), 0 if the lines or the grid are too large; and the launch (tables and
+// consts as above).
+int tri2d_fused_lines(int prec, int64_t nx, int64_t n1, int64_t nchunks);
+cudaError_t launch_tri2d_fused(int prec, int step, const void* fhat, const void* faces, const void* tables, void* out,
+                               void* partial, const Solve2DArgs& a, const int* skip, cudaStream_t st, Profiler* prof,
+                               const void* consts);
 size_t chunk_record_bytes(int prec);
 // Boundary faces from the partials, v[face][ix] = s_face * sum partial (complex
 // scales, face 0 then 1), then out = C_bb (v + prev) (prev may be null): C_bb
