@@ -39,6 +39,9 @@ struct Plane3DArgs {
   double en_o[2], eninv_o[2], g_o[2], ginv_o[2];
   double en_i[2], eninv_i[2], g_i[2], ginv_i[2];
   double mden;  // mass matrix denominator (MassCoef): 6 the paper's elements, 12 the modified ones
+  // derived on the host (a division is a dozen FP64 instructions of a thread)
+  MassCoef mx, mz;
+  double rhx, rhz, rny, rnz;  // 1/hx, 1/hz, 1/ny, 1/nz
 };
 
 constexpr int XC = 32;  // rows per reduction chunk
@@ -79,8 +82,13 @@ struct ThomasRow {
 //   D11 = (1 + i w hz)/hz - p hz/3, D1n = -1/hz - p hz/6, E11 = hz/3, E1n = hz/6,
 // M, K along x; p = w^2 - Lam_{1,l} (complex for outer A modes).
 template <typename C>
-__device__ void plane_cbb(const C* v, const C* w2, C* out, int nx, double hx, double hz, double wx, double wz,
-                          double pre, double pim, C g, C ginv, double mden) {
+__device__ void plane_cbb(const C* v, const C* w2, C* out, const Plane3DArgs& a, double pre, double pim) {
+  using R = decltype(C().x);
+  const int nx = (int)a.nx;
+  const R mo = (R)a.mx.off, ko = (R)(-a.rhx), E11 = (R)a.mz.end, E1n = (R)a.mz.off;
+  const C D11 = mk<C>(a.rhz - pre * a.mz.end, a.wz - pim * a.mz.end);
+  const C D1n = mk<C>(-a.rhz - pre * a.mz.off, -pim * a.mz.off);
+  const C g = mk<C>(a.g_i[0], a.g_i[1]), ginv = mk<C>(a.ginv_i[0], a.ginv_i[1]);
   for (int ix = threadIdx.x; ix < nx; ix += blockDim.x) {
     auto get = [&](int face, int j) -> C {
       C t = v[face * nx + j];
@@ -88,21 +96,17 @@ __device__ void plane_cbb(const C* v, const C* w2, C* out, int nx, double hx, do
       return t;
     };
     const bool end = (ix == 0 || ix == nx - 1);
-    const MassCoef mc = mass_coef(hx, mden), mcz = mass_coef(hz, mden);
-    const double md = end ? mc.end : mc.in, mo = mc.off;
-    const double kdr = end ? 1.0 / hx : 2.0 / hx, kdi = end ? -wx : 0.0, ko = -1.0 / hx;
+    const R md = (R)(end ? a.mx.end : a.mx.in);
+    const C kd = end ? mk<C>(a.rhx, -a.wx) : mk<C>(2.0 * a.rhx, 0.0);
     C Mv[2], Kv[2];
     for (int f = 0; f < 2; ++f) {
       C v0 = get(f, ix);
       C vm = ix > 0 ? get(f, ix - 1) : mk<C>(0, 0);
       C vp = ix < nx - 1 ? get(f, ix + 1) : mk<C>(0, 0);
       C nb = cadd(vm, vp);
-      Mv[f] = cadd(cscale(v0, (decltype(v0.x))md), cscale(nb, (decltype(v0.x))mo));
-      Kv[f] = cadd(cmul(v0, mk<C>(kdr, kdi)), cscale(nb, (decltype(v0.x))ko));
+      Mv[f] = cadd(cscale(v0, md), cscale(nb, mo));
+      Kv[f] = cadd(cmul(v0, kd), cscale(nb, ko));
     }
-    const C D11 = mk<C>(1.0 / hz - pre * mcz.end, wz - pim * mcz.end);
-    const C D1n = mk<C>(-1.0 / hz - pre * mcz.off, -pim * mcz.off);
-    const auto E11 = (decltype(D11.x))mcz.end, E1n = (decltype(D11.x))mcz.off;
     out[ix] = cadd(cadd(cmul(D11, Mv[0]), cscale(Kv[0], E11)), cmul(ginv, cadd(cmul(D1n, Mv[1]), cscale(Kv[1], E1n))));
     out[nx + ix] = cadd(cmul(g, cadd(cmul(D1n, Mv[0]), cscale(Kv[0], E1n))), cadd(cmul(D11, Mv[1]), cscale(Kv[1], E11)));
   }
@@ -266,7 +270,7 @@ __global__ void __launch_bounds__(1024) k_plane3d(const typename cpx<T>::type* _
         sn = ac ? cmul(x, twm) : mk<C>(0, 0);
       },
       vin, mk<C>(1.0 / (double)nz, 0), mk<C>(a.en_i[0] / (double)nz, a.en_i[1] / (double)nz));
-  plane_cbb(vin, (const C*)nullptr, cin, nx, a.hx, a.hz, a.wx, a.wz, pre, pim, gi, giv, a.mden);
+  plane_cbb(vin, (const C*)nullptr, cin, a, pre, pim);
   __syncthreads();
   // inner Step 2: A solve on the generated rhs, reduce to w_in
   forward(thA, tabA, [&](int ix) { return cadd(cin[ix], cscale(cin[nx + ix], pari)); });
@@ -278,7 +282,7 @@ __global__ void __launch_bounds__(1024) k_plane3d(const typename cpx<T>::type* _
         sn = cscale(t, pari);
       },
       win, mk<C>(1, 0), mk<C>(1, 0));
-  plane_cbb(vin, win, cin, nx, a.hx, a.hz, a.wx, a.wz, pre, pim, gi, giv, a.mden);
+  plane_cbb(vin, (const C*)win, cin, a, pre, pim);
   __syncthreads();
   // inner Step 3: corrected B-aux solve, y3 written over the scratch
   forward(thB, tabB, [&](int ix) {
@@ -313,32 +317,44 @@ __global__ void __launch_bounds__(1024) k_plane3d(const typename cpx<T>::type* _
 //   out[face][x][m] = sum_l wgt_face(l) * y3(x, l, m)
 // step 1: wgt = (1/ny, e^{-2 pi i l/ny}/ny); step 2: wgt = (sigma_l, par_l sigma_l).
 // The weights of a run of outer modes are staged in shared memory in the
-// compute precision; each thread sums over l in order, loading kOuterBatch
-// values ahead of the dependent sums.
+// compute precision; SPLIT threads share an output's modes, each summing a
+// contiguous part of every run in order, loading kOuterBatch values ahead of
+// the dependent sums, and the parts are added in order at the end.  par_l is
+// +-1 (the parity of mode l), so Step 2 keeps the sums of the two parities and
+// forms s1 and sn from them: 4 multiply-adds per value instead of 8 operations.
+//
+// Bound: memory for large faces (512^3 complex64: y3 once in 0.19 ms of 0.16);
+// for small ones the chain of loads of one thread, hence SPLIT = 4 while the
+// faces give fewer than kOuterSplitBelow threads (190 x 223 x 127 complex64: 40 us, now 25); the
+// FP64 pipe in complex128 (201 x 150 x 175: 94 us, now 88).
 constexpr int kOuterChunk = 1024;
 constexpr int kOuterBatch = 8;
-template <typename T, int OSTEP>
+constexpr int64_t kOuterSplitBelow = 152 * 1024;
+template <typename T, int OSTEP, int SPLIT>
 __global__ void __launch_bounds__(256) k_reduce_outer(const typename cpx<T>::type* __restrict__ y3,
                                                       typename cpx<T>::type* __restrict__ out, Plane3DArgs a,
                                                       const int* __restrict__ skip) {
   using C = typename cpx<T>::type;
+  constexpr int NO = 256 / SPLIT;  // outputs of a block
   if (skip && *skip) return;  // uniform over the grid
   __shared__ C sw[kOuterChunk];
   __shared__ T sp[OSTEP == 2 ? kOuterChunk : 1];
+  __shared__ C part[SPLIT > 1 ? 2 * 256 : 1];
   const int64_t ny = a.ny, nz = a.nz;
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int o = threadIdx.x % NO, q = threadIdx.x / NO;
+  const int64_t i = (int64_t)blockIdx.x * NO + o;
   const bool act = i < a.nx * nz;
   const int64_t ix = act ? i / nz : 0, m = act ? i - ix * nz : 0;
   const C* src = y3 + ix * ny * nz + m;
-  C s1 = mk<C>(0, 0), sn = mk<C>(0, 0);
+  C s1 = mk<C>(0, 0), sn = mk<C>(0, 0);  // Step 2: sums of the parities +1, -1
   auto add = [&](C v, int j) {
     if (OSTEP == 1) {
       s1 = cadd(s1, v);
-      sn = cadd(sn, cmul(v, sw[j]));
+      sn = cfma(v, sw[j], sn);
+    } else if (sp[j] > T(0)) {
+      s1 = cfma(v, sw[j], s1);
     } else {
-      const C t = cmul(v, sw[j]);
-      s1 = cadd(s1, t);
-      sn = cadd(sn, cscale(t, sp[j]));
+      sn = cfma(v, sw[j], sn);
     }
   };
   for (int64_t l0 = 0; l0 < ny; l0 += kOuterChunk) {
@@ -355,21 +371,38 @@ __global__ void __launch_bounds__(256) k_reduce_outer(const typename cpx<T>::typ
     }
     __syncthreads();
     if (act) {
-      int j = 0;
-      for (; j + kOuterBatch <= cnt; j += kOuterBatch) {
+      const int len = (cnt + SPLIT - 1) / SPLIT;
+      int j = q * len;
+      const int j1 = min(cnt, j + len);
+      for (; j + kOuterBatch <= j1; j += kOuterBatch) {
         C v[kOuterBatch];
 #pragma unroll
-        for (int q = 0; q < kOuterBatch; ++q) v[q] = src[(l0 + j + q) * nz];
+        for (int t = 0; t < kOuterBatch; ++t) v[t] = src[(l0 + j + t) * nz];
 #pragma unroll
-        for (int q = 0; q < kOuterBatch; ++q) add(v[q], j + q);
+        for (int t = 0; t < kOuterBatch; ++t) add(v[t], j + t);
       }
-      for (; j < cnt; ++j) add(src[(l0 + j) * nz], j);
+      for (; j < j1; ++j) add(src[(l0 + j) * nz], j);
+    }
+  }
+  if (SPLIT > 1) {
+    part[threadIdx.x] = s1;
+    part[256 + threadIdx.x] = sn;
+    __syncthreads();
+    if (q > 0) return;
+#pragma unroll
+    for (int t = 1; t < SPLIT; ++t) {
+      s1 = cadd(s1, part[t * NO + o]);
+      sn = cadd(sn, part[256 + t * NO + o]);
     }
   }
   if (!act) return;
   if (OSTEP == 1) {
-    s1 = cscale(s1, (decltype(s1.x))(1.0 / (double)ny));
-    sn = cmul(sn, mk<C>(a.en_o[0] / (double)ny, a.en_o[1] / (double)ny));
+    s1 = cscale(s1, (T)a.rny);
+    sn = cmul(sn, mk<C>(a.en_o[0] * a.rny, a.en_o[1] * a.rny));
+  } else {
+    const C e = s1;
+    s1 = cadd(e, sn);
+    sn = csub(e, sn);
   }
   out[i] = s1;
   out[a.nx * nz + i] = sn;
@@ -380,58 +413,90 @@ __global__ void __launch_bounds__(256) k_reduce_outer(const typename cpx<T>::typ
 //   c_1 = (hy/3) S v_1 + ((1 + i w hy)/hy) P v_1 + g^-1 [(hy/6) S v_n - (1/hy) P v_n],
 //   c_n = g [(hy/6) S v_1 - (1/hy) P v_1] + (hy/3) S v_n + ((1 + i w hy)/hy) P v_n,
 // g the wrap factor of the gamma-circulant auxiliary (1: periodic).
+//
+// The entries of S and P depend on where (x, z) lies only through "end of the
+// axis, inside, or a neighbour" of either axis: nine of each, formed on the
+// host in FP64 (in the kernel, with its
+// FP64 divisions, they cost about 80 us a launch at 512^3).
+template <typename C>
+struct OuterCbb {
+  C s[3][3];                  // [x: end, inside, neighbour][z: the same]
+  decltype(C().x) p[3][3];
+  decltype(C().x) e11, e1n, d1n;
+  C d11, g, gv;
+};
+
+template <typename C>
+OuterCbb<C> outer_cbb_consts(const Plane3DArgs& a) {
+  using R = decltype(C().x);
+  auto ent = [&](double h, double w, int kind, double& m, double& kr, double& ki) {
+    const MassCoef mc = mass_coef(h, a.mden);
+    m = kind == 0 ? mc.end : kind == 1 ? mc.in : mc.off;
+    kr = (kind == 0 ? 1.0 : kind == 1 ? 2.0 : -1.0) / h;
+    ki = kind == 0 ? -w : 0.0;
+  };
+  OuterCbb<C> k;
+  const double w2 = a.omega * a.omega;
+  auto put = [](double x, double y) {
+    C c;
+    c.x = (R)x;
+    c.y = (R)y;
+    return c;
+  };
+  for (int x = 0; x < 3; ++x)
+    for (int z = 0; z < 3; ++z) {
+      double mx, kxr, kxi, mz, kzr, kzi;
+      ent(a.hx, a.wx, x, mx, kxr, kxi);
+      ent(a.hz, a.wz, z, mz, kzr, kzi);
+      k.s[x][z] = put(kxr * mz + mx * kzr - w2 * mx * mz, kxi * mz + mx * kzi);
+      k.p[x][z] = (R)(mx * mz);
+    }
+  const MassCoef my = mass_coef(a.hy, a.mden);
+  k.e11 = (R)my.end;
+  k.e1n = (R)my.off;
+  k.d1n = (R)(-1.0 / a.hy);
+  k.d11 = put(1.0 / a.hy, a.wy);
+  k.g = put(a.g_o[0], a.g_o[1]);
+  k.gv = put(a.ginv_o[0], a.ginv_o[1]);
+  return k;
+}
+
 template <typename T>
 __global__ void k_outer_cbb(const typename cpx<T>::type* __restrict__ v, const typename cpx<T>::type* __restrict__ w,
-                            typename cpx<T>::type* __restrict__ out, Plane3DArgs a, const int* __restrict__ skip) {
+                            typename cpx<T>::type* __restrict__ out, int64_t nx, int64_t nz,
+                            OuterCbb<typename cpx<T>::type> k, const int* __restrict__ skip) {
   using C = typename cpx<T>::type;
   if (skip && *skip) return;
-  const int64_t nx = a.nx, nz = a.nz;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nx * nz) return;
   const int64_t ix = i / nz, iz = i - ix * nz;
-  auto ent = [&](int64_t n, double h, double w, int64_t j, int d, double& m, double& kr, double& ki) {
-    const bool end = (j == 0 || j == n - 1);
-    const MassCoef mc = mass_coef(h, a.mden);
-    if (d == 0) {
-      m = end ? mc.end : mc.in;
-      kr = (end ? 1.0 : 2.0) / h;
-      ki = end ? -w : 0.0;
-    } else {
-      m = mc.off;
-      kr = -1.0 / h;
-      ki = 0.0;
-    }
-  };
+  const int xin = (ix == 0 || ix == nx - 1) ? 0 : 1, zin = (iz == 0 || iz == nz - 1) ? 0 : 1;
   C Sv[2] = {mk<C>(0, 0), mk<C>(0, 0)}, Pv[2] = {mk<C>(0, 0), mk<C>(0, 0)};
-  const double w2 = a.omega * a.omega;
+#pragma unroll
   for (int dx = -1; dx <= 1; ++dx) {
     const int64_t jx = ix + dx;
     if (jx < 0 || jx >= nx) continue;
-    double mx, kxr, kxi;
-    ent(nx, a.hx, a.wx, ix, dx, mx, kxr, kxi);
+#pragma unroll
     for (int dz = -1; dz <= 1; ++dz) {
       const int64_t jz = iz + dz;
       if (jz < 0 || jz >= nz) continue;
-      double mz, kzr, kzi;
-      ent(nz, a.hz, a.wz, iz, dz, mz, kzr, kzi);
-      const C cs = mk<C>(kxr * mz + mx * kzr - w2 * mx * mz, kxi * mz + mx * kzi);
-      const auto cp = (decltype(cs.x))(mx * mz);
+      // selected, not indexed: the entries stay in the constant bank
+      const C cs = dx ? (dz ? k.s[2][2] : zin ? k.s[2][1] : k.s[2][0])
+                      : (dz ? (xin ? k.s[1][2] : k.s[0][2])
+                            : xin ? (zin ? k.s[1][1] : k.s[1][0]) : (zin ? k.s[0][1] : k.s[0][0]));
+      const T cp = dx ? (dz ? k.p[2][2] : zin ? k.p[2][1] : k.p[2][0])
+                      : (dz ? (xin ? k.p[1][2] : k.p[0][2])
+                            : xin ? (zin ? k.p[1][1] : k.p[1][0]) : (zin ? k.p[0][1] : k.p[0][0]));
       for (int f = 0; f < 2; ++f) {
         C t = v[f * nx * nz + jx * nz + jz];
         if (w) t = cadd(t, w[f * nx * nz + jx * nz + jz]);
-        Sv[f] = cadd(Sv[f], cmul(cs, t));
+        Sv[f] = cfma(cs, t, Sv[f]);
         Pv[f] = cadd(Pv[f], cscale(t, cp));
       }
     }
   }
-  using T2 = decltype(Sv[0].x);
-  const MassCoef mcy = mass_coef(a.hy, a.mden);
-  const T2 e11 = (T2)mcy.end, e1n = (T2)mcy.off;
-  const C d11 = mk<C>(1.0 / a.hy, a.wy);
-  const T2 d1n = (T2)(-1.0 / a.hy);
-  const C g = mk<C>(a.g_o[0], a.g_o[1]), gv = mk<C>(a.ginv_o[0], a.ginv_o[1]);
-  out[i] = cadd(cadd(cscale(Sv[0], e11), cmul(d11, Pv[0])), cmul(gv, cadd(cscale(Sv[1], e1n), cscale(Pv[1], d1n))));
-  out[nx * nz + i] = cadd(cmul(g, cadd(cscale(Sv[0], e1n), cscale(Pv[0], d1n))), cadd(cscale(Sv[1], e11), cmul(d11, Pv[1])));
+  out[i] = cadd(cadd(cscale(Sv[0], k.e11), cmul(k.d11, Pv[0])), cmul(k.gv, cadd(cscale(Sv[1], k.e1n), cscale(Pv[1], k.d1n))));
+  out[nx * nz + i] = cadd(cmul(k.g, cadd(cscale(Sv[0], k.e1n), cscale(Pv[0], k.d1n))), cadd(cscale(Sv[1], k.e11), cmul(k.d11, Pv[1])));
 }
 
 // Reciprocal pivots of the inner tridiagonal lines of one line type (outer
@@ -523,6 +588,12 @@ Plane3DArgs make_args(const Plan3D& p) {
   a.wy = p.wc[1];
   a.wz = p.wc[2];
   a.mden = p.mden;
+  a.mx = mass_coef(a.hx, a.mden);
+  a.mz = mass_coef(a.hz, a.mden);
+  a.rhx = 1.0 / a.hx;
+  a.rhz = 1.0 / a.hz;
+  a.rny = 1.0 / (double)a.ny;
+  a.rnz = 1.0 / (double)a.nz;
   a.lamBo = p.axo->lamB;
   a.invmuo = p.axo->invmu;
   a.lamAo = p.axo->lamA;
@@ -1325,10 +1396,11 @@ __global__ void __launch_bounds__(256) k_inner_reduce(InnerArgs ia, const typena
   C* sw = sv + 2 * nx;                     // [2][nx] w_in
   C* vwl = vw + l * 4 * nx;                // [v_in 2 nx][w_in 2 nx]
   const C* pp = part + l * (int64_t)ia.nparts * 2 * nx;
-  const C sc1 = ISTEP == 1 ? mk<C>(1.0 / (double)a.nz, 0) : mk<C>(1, 0);
-  const C scn = ISTEP == 1 ? mk<C>(a.en_i[0] / (double)a.nz, a.en_i[1] / (double)a.nz) : mk<C>(1, 0);
+  const C sc1 = ISTEP == 1 ? mk<C>(a.rnz, 0) : mk<C>(1, 0);
+  const C scn = ISTEP == 1 ? mk<C>(a.en_i[0] * a.rnz, a.en_i[1] * a.rnz) : mk<C>(1, 0);
   for (int e = threadIdx.x; e < 2 * nx; e += blockDim.x) {
     C acc = mk<C>(0, 0);
+#pragma unroll 4
     for (int q = 0; q < ia.nparts; ++q) acc = cadd(acc, pp[(int64_t)q * 2 * nx + e]);
     if (roff)  // lines of this plane solved in FP64, in route order
       for (int q = roff[l]; q < roff[l + 1]; ++q) acc = cadd(acc, rpart[(int64_t)q * 2 * nx + e]);
@@ -1346,8 +1418,7 @@ __global__ void __launch_bounds__(256) k_inner_reduce(InnerArgs ia, const typena
   const double lo_re = OSTEP == 2 ? a.lamAo[2 * l] : a.lamBo[2 * l];
   const double lo_im = OSTEP == 2 ? a.lamAo[2 * l + 1] : a.lamBo[2 * l + 1];
   const double pre = a.omega * a.omega - lo_re, pim = -lo_im;
-  plane_cbb(sv, ISTEP == 2 ? (const C*)sw : (const C*)nullptr, cin + l * 2 * nx, nx, a.hx, a.hz, a.wx, a.wz, pre, pim,
-            mk<C>(a.g_i[0], a.g_i[1]), mk<C>(a.ginv_i[0], a.ginv_i[1]), a.mden);
+  plane_cbb(sv, ISTEP == 2 ? (const C*)sw : (const C*)nullptr, cin + l * 2 * nx, a, pre, pim);
 }
 
 template <typename T>
@@ -1452,10 +1523,13 @@ template <typename T>
 cudaError_t launch_reduce_outer(int ostep, const Plan3D& p, void* out, const int* skip, cudaStream_t st) {
   using C = typename cpx<T>::type;
   const int bs = 256;
-  const unsigned grid = (unsigned)((p.n[0] * p.n[2] + bs - 1) / bs);
+  const int64_t no = p.n[0] * p.n[2];
+  const int split = no < kOuterSplitBelow ? 4 : 1;
+  const unsigned grid = (unsigned)((no * split + bs - 1) / bs);
   Plane3DArgs a = make_args(p);
-  if (ostep == 1) k_reduce_outer<T, 1><<<grid, bs, 0, st>>>((const C*)p.dbuf, (C*)out, a, skip);
-  else k_reduce_outer<T, 2><<<grid, bs, 0, st>>>((const C*)p.dbuf, (C*)out, a, skip);
+  auto kern = split == 4 ? (ostep == 1 ? k_reduce_outer<T, 1, 4> : k_reduce_outer<T, 2, 4>)
+                         : (ostep == 1 ? k_reduce_outer<T, 1, 1> : k_reduce_outer<T, 2, 1>);
+  kern<<<grid, bs, 0, st>>>((const C*)p.dbuf, (C*)out, a, skip);
   return cudaGetLastError();
 }
 
@@ -1464,7 +1538,8 @@ cudaError_t launch_outer_cbb(const Plan3D& p, const void* v, const void* w, void
   using C = typename cpx<T>::type;
   const int bs = 256;
   const unsigned grid = (unsigned)((p.n[0] * p.n[2] + bs - 1) / bs);
-  k_outer_cbb<T><<<grid, bs, 0, st>>>((const C*)v, (const C*)w, (C*)out, make_args(p), skip);
+  k_outer_cbb<T><<<grid, bs, 0, st>>>((const C*)v, (const C*)w, (C*)out, p.n[0], p.n[2],
+                                    outer_cbb_consts<C>(make_args(p)), skip);
   return cudaGetLastError();
 }
 
