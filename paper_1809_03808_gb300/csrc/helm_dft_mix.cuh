@@ -67,7 +67,7 @@ __device__ __forceinline__ void store_many(void* p, int mode, int64_t g0, int of
 #pragma unroll
     for (int q = 0; q < R; ++q) {
       if (q >= hi) break;
-      if (q >= lo) o[off + q * doff] = make_double2((double)v[q].x, (double)v[q].y);
+      if (q >= lo) o[off + q * doff] = make_double2(widen(v[q].x), widen(v[q].y));
     }
   } else if (mode == kOutAccumC128) {
     double2* o = reinterpret_cast<double2*>(p) + g0;
@@ -81,8 +81,8 @@ __device__ __forceinline__ void store_many(void* p, int mode, int64_t g0, int of
 #pragma unroll
       for (int i = 0; i < kAccumBatch; ++i)
         if (q0 + i < R && q0 + i >= lo && q0 + i < hi)
-          o[off + (q0 + i) * doff] = make_double2(u[i].x + accum_scale * (double)v[(q0 + i) % R].x,
-                                                  u[i].y + accum_scale * (double)v[(q0 + i) % R].y);
+          o[off + (q0 + i) * doff] = make_double2(u[i].x + accum_scale * widen(v[(q0 + i) % R].x),
+                                                  u[i].y + accum_scale * widen(v[(q0 + i) % R].y));
     }
   } else if (mode == kOutFF) {
     float4* o = reinterpret_cast<float4*>(p) + g0;

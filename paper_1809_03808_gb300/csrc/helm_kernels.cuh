@@ -34,6 +34,16 @@ __device__ __forceinline__ C cvt(S s) {
   c.y = (decltype(c.y))s.y;
   return c;
 }
+// (double)x.  The conversion instruction runs on the FP64 pipe (16 clocks per
+// warp); for normal numbers the exponent is rebiased (127 -> 1023) and the
+// fraction shifted on the integer pipes instead.  Zeros, denormals, infinities
+// and NaNs are converted.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t b = __float_as_uint(x), m = b & 0x7fffffffu;
+  if (m - 0x00800000u >= 0x7f000000u) return (double)x;
+  return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(m << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
 template <typename C>
 __device__ __forceinline__ C cadd(C a, C b) {
   a.x += b.x;

@@ -323,7 +323,8 @@ __global__ void __launch_bounds__(1024) k_plane3d(const typename cpx<T>::type* _
 // +-1 (the parity of mode l), so Step 2 keeps the sums of the two parities and
 // forms s1 and sn from them: 4 multiply-adds per value instead of 8 operations.
 //
-// Bound: memory for large faces (512^3 complex64: y3 once in 0.19 ms of 0.16);
+// Bound: memory for large faces (512^3 complex64: y3 once, 0.16 ms at the copy
+// rate, takes 0.18);
 // for small ones the chain of loads of one thread, hence SPLIT = 4 while the
 // faces give fewer than kOuterSplitBelow threads (190 x 223 x 127 complex64: 40 us, now 25); the
 // FP64 pipe in complex128 (201 x 150 x 175: 94 us, now 88).
