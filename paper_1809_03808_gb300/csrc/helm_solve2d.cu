@@ -238,18 +238,21 @@ __global__ void __launch_bounds__(128) k_tri_pass1(const typename cpx<T>::type* 
 // q_k = -b we_k (stored in rec.we).  A block takes carry_lines() lines (one per
 // x thread, so every load of a field is a contiguous run of lines) and splits
 // their chunks into blockDim.y contiguous segments (one per y thread).  Each
-// thread composes the maps of its segment, one thread per line folds the
-// segment maps in shared memory into each segment's incoming carry, and each
-// thread then runs its segment's recurrence from that carry.  Same recurrences
-// as the sequential scan, regrouped once, in the precision of the records.
+// thread composes the maps of its segment, the segment maps are folded in
+// shared memory into each segment's incoming carry, and each thread then runs
+// its segment's recurrence from that carry.  Same recurrences as the sequential
+// scan, regrouped once, in the precision of the records.
 //
 // Bound, complex128: the FP64 pipe (2 fused multiply-adds per clock and SM, so
 // one instruction of a warp takes 16 clocks however few of its lanes work).
-// The fold is therefore done once per line by half a warp (a chain of <= 31
-// steps of 4 fused operations) and not by every segment for itself, which
-// took 16 warps x 15 steps on average: at 129^2 that was most of 39 us, now
-// 16 (with the timing's own 4-5); at 8192 x 4096 418 us, now 283.  Segments hold at least
-// kCarryMinSeg chunks, so that short lines neither fold nor launch empty ones.
+// The fold is therefore done once per line by one row of threads (a chain of
+// <= 31 steps of 4 fused operations) and not by every segment for itself, which
+// took 16 warps x 15 steps on average: at 129^2 that was most of 39 us, now 16
+// (with the timing's own 4-5); at 8192 x 4096 418 us, now 283.  In complex64
+// every segment folds its own prefix, which is free beside the barrier it saves
+// (8192 x 4096: 33 us a launch against 40).  Segments hold at least kCarryMinSeg
+// chunks, so that short lines neither fold nor launch empty ones.
+//
 // 128 bytes of lines, so that every load of a field is whole lines of memory
 template <typename T>
 __host__ __device__ constexpr int carry_lines() {
@@ -294,6 +297,7 @@ __global__ void __launch_bounds__(carry_lines<T>() * kCarrySeg, 2)
     k_tri_carry(RecSoA<typename cpx<T>::type> rec, int64_t n1, int64_t K, const int* __restrict__ skip) {
   using C = typename cpx<T>::type;
   constexpr int B = carry_batch<T>(), NL = carry_lines<T>();
+  constexpr bool F64 = sizeof(T) == 8;
   if (skip && *skip) return;  // uniform over the grid
   __shared__ C shC[kCarrySeg][NL], shP[kCarrySeg][NL];
   const int lx = threadIdx.x, sg = threadIdx.y, nseg = blockDim.y;
@@ -324,9 +328,14 @@ __global__ void __launch_bounds__(carry_lines<T>() * kCarrySeg, 2)
   shC[sg][lx] = A;
   shP[sg][lx] = P;
   __syncthreads();
-  if (sg == 0) carry_fold<C, NL>(shC, shP, lx, nseg, 1);
-  __syncthreads();
-  C Y = shC[sg][lx];
+  C Y = zero;
+  if (F64) {
+    if (sg == 0) carry_fold<C, NL>(shC, shP, lx, nseg, 1);
+    __syncthreads();
+    Y = shC[sg][lx];
+  } else {
+    for (int g = 0; g < sg; ++g) Y = cfma(shP[g][lx], Y, shC[g][lx]);
+  }
   // forward recurrence; c_k replaces bsum_k
   if (act)
     for (int64_t kb = k0; kb < k1; kb += B) {
@@ -373,9 +382,14 @@ __global__ void __launch_bounds__(carry_lines<T>() * kCarrySeg, 2)
   shC[sg][lx] = Cs;
   shP[sg][lx] = Q;
   __syncthreads();
-  if (sg == 0) carry_fold<C, NL>(shC, shP, lx, nseg, -1);
-  __syncthreads();
-  C X = shC[sg][lx];
+  C X = zero;
+  if (F64) {
+    if (sg == 0) carry_fold<C, NL>(shC, shP, lx, nseg, -1);
+    __syncthreads();
+    X = shC[sg][lx];
+  } else {
+    for (int g = nseg - 1; g > sg; --g) X = cfma(shP[g][lx], X, shC[g][lx]);
+  }
   if (act)
     for (int64_t kb = k1 - 1; kb >= k0; kb -= B) {
       C cv[B], qv[B];
