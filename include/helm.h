@@ -210,10 +210,11 @@ int helm_set_precision_routing(helm_plan_t p, double tau);
 /* Kernel variants (the autotuner's choices; the paper fixes none of them).
  * Every variant computes the same solution; they differ in speed by grid.
  *   HELM_VARIANT_INNER_CHUNK  3D: rows per chunk of the tiled inner sweeps
- *                             (8, 16 or 32; default 16, 32 for lines beyond
- *                             1024 rows, 512 in complex128).
+ *                             (8, 16 or 32; default 16; 32 for lines beyond
+ *                             256 rows in complex64, and where 16 would be
+ *                             too many chunks for a CTA).
  *   HELM_VARIANT_INNER_TILES  3D: tiles of 16 inner modes per CTA (1..8;
- *                             default 1..4 by grid size).
+ *                             default 1, 2 on large complex64 grids).
  *   HELM_VARIANT_TRI2D        2D complex64: 0 = one kernel per step on grids
  *                             of up to 4 Mi unknowns and 2048 rows, beyond
  *                             them bulk-copy fed passes where the x1 length
