@@ -33,6 +33,7 @@
 #include <cmath>
 
 #include "helm_async.cuh"
+#include "helm_fx.h"
 #include "helm_kernels.cuh"
 #include "helm_resid.h"
 
@@ -42,16 +43,13 @@ namespace {
 
 typedef long long ll;
 
-struct Limb {
-  int h, l;
-};
 struct FxArgs {
   int nx, ny, nz;
   int es;  // eS
-  // the coefficients' negatives: real ones inside (class 0), then all classes (re, im)
+  // the coefficients' negatives: real ones inside (class 0), then all classes
   Limb q[4], r[4];
-  Limb c0[8][4][2];
-  Limb c1[4][4][2];
+  LimbC c0[8][4];
+  LimbC c1[4][4];
 };
 
 constexpr int kBadKey = 1 << 20;  // key of a NaN or an infinity
@@ -140,19 +138,17 @@ __device__ __forceinline__ void dot_real(const cll (&P)[NK], const Limb* q, cons
 // s + sum_k c_k P_k with complex coefficients c_k = (re, im); the products
 // with the real and with the imaginary parts have a middle sum each (its bound)
 template <int NK>
-__device__ __forceinline__ cll dot_cplx(cll s, const cll (&P)[NK], const Limb (*c)[2]) {
+__device__ __forceinline__ cll dot_cplx(cll s, const cll (&P)[NK], const LimbC* c) {
   ll ax = kHalf, ay = kHalf, bx = kHalf, by = kHalf;
 #pragma unroll
   for (int k = 0; k < NK; ++k) {
     int xh, xl, yh, yl;
     split32(P[k].x, xh, xl);
     split32(P[k].y, yh, yl);
-    const Limb re = c[k][0], im = c[k][1];
-    const Limb nim = {-im.h, -im.l};
-    mac(s.x, ax, xh, xl, re);
-    mac(s.x, bx, yh, yl, nim);
-    mac(s.y, ay, yh, yl, re);
-    mac(s.y, by, xh, xl, im);
+    mac(s.x, ax, xh, xl, c[k].re);
+    mac(s.x, bx, yh, yl, c[k].nim);
+    mac(s.y, ay, yh, yl, c[k].re);
+    mac(s.y, by, xh, xl, c[k].im);
   }
   return {fold(fold(s.x, ax), bx), fold(fold(s.y, ay), by)};
 }
@@ -497,22 +493,12 @@ FxArgs fx_args(int dim, const ResidQArgs& q) {
   }
   if (!std::isfinite(S) || S <= 0) S = 1;
   std::frexp(S * (1 + 1e-12), &a.es);  // S < 2^es
-  auto limb = [&](double v) -> Limb {
-    const long long c = std::isfinite(v) ? std::llround(std::ldexp(-v, 62 - a.es)) : 0;
-    const long long h = (c + (1ll << 31)) >> 32;
-    return {(int)h, (int)(c - (h << 32))};
-  };
+  auto neg = [&](double2 c) { return fx_limb_c(-c.x, -c.y, a.es); };
   for (int k = 0; k < nk; ++k) {
-    a.q[k] = limb(q.c0[0][k].x);
-    a.r[k] = limb(q.c1[0][k].x);
-    for (int c = 0; c < n0; ++c) {
-      a.c0[c][k][0] = limb(q.c0[c][k].x);
-      a.c0[c][k][1] = limb(q.c0[c][k].y);
-    }
-    for (int c = 0; c < n1; ++c) {
-      a.c1[c][k][0] = limb(q.c1[c][k].x);
-      a.c1[c][k][1] = limb(q.c1[c][k].y);
-    }
+    a.q[k] = neg(q.c0[0][k]).re;
+    a.r[k] = neg(q.c1[0][k]).re;
+    for (int c = 0; c < n0; ++c) a.c0[c][k] = neg(q.c0[c][k]);
+    for (int c = 0; c < n1; ++c) a.c1[c][k] = neg(q.c1[c][k]);
   }
   return a;
 }
