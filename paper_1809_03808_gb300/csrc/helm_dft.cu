@@ -31,6 +31,7 @@ bool dft_supported(const DftPlan& p, size_t elem_bytes, int max_smem) {
     const int64_t m = bluestein_length(p.n);
     return m <= 8192 && (size_t)2 * m * elem_bytes <= (size_t)max_smem;
   }
+  // two bare lines: all that the row kernels need (they pad them where there is room)
   return (size_t)2 * p.n * elem_bytes <= (size_t)max_smem;
 }
 

@@ -114,11 +114,14 @@ __device__ __forceinline__ void store_many(void* p, int mode, int64_t g0, int of
 // What the passes of one CTA share.  Lines: ROWS, `lines` lines of m.n points
 // [line][padded point] (a padding point per 128 bytes keeps the strided writes
 // of a pass off each other's banks); columns, 2^lt neighbouring columns
-// [point][column], the lanes of a warp on consecutive columns.
-template <typename T, bool COLS, bool BS>
+// [point][column], the lanes of a warp on consecutive columns.  TIGHT: rows
+// without padding, see run_mix.
+template <typename T, bool COLS, bool BS, bool TIGHT>
 struct Ctx {
   using C = typename cpx<T>::type;
-  static constexpr int kPad = sizeof(T) == 4 ? 4 : 3;
+  static constexpr int kPad = TIGHT ? 31 : sizeof(T) == 4 ? 4 : 3;
+  // points from one line to the next
+  static __host__ __device__ constexpr int pitch_of(int n) { return TIGHT ? n : n + (n >> kPad) + 1; }
   const void* in;
   void* out;
   int kind;      // of `in` (kIn*)
@@ -243,8 +246,8 @@ struct Ctx {
 };
 
 // One pass of radix R <= 10: thread per butterfly.
-template <int R, typename T, bool COLS, bool BS>
-__device__ __forceinline__ void pass_reg(const Ctx<T, COLS, BS>& x, const MixStage& st, int s, bool last, bool mid) {
+template <int R, typename T, bool COLS, bool BS, bool TIGHT>
+__device__ __forceinline__ void pass_reg(const Ctx<T, COLS, BS, TIGHT>& x, const MixStage& st, int s, bool last, bool mid) {
   using C = typename cpx<T>::type;
   const int total = x.items(st.nb);
   const C* src = x.buf(s + 1);
@@ -287,8 +290,8 @@ __device__ __forceinline__ void pass_reg(const Ctx<T, COLS, BS>& x, const MixSta
 // Bluestein: the convolution's first len points (in buf) to global memory.
 // The last pass does not store them itself: with the lines ending inside its
 // butterflies, their bounds cost more registers than this exchange's time.
-template <typename T, bool COLS, bool BS>
-__device__ __forceinline__ void copy_out(const Ctx<T, COLS, BS>& x, const typename cpx<T>::type* buf) {
+template <typename T, bool COLS, bool BS, bool TIGHT>
+__device__ __forceinline__ void copy_out(const Ctx<T, COLS, BS, TIGHT>& x, const typename cpx<T>::type* buf) {
   using C = typename cpx<T>::type;
   const int dk = COLS ? (int)blockDim.x >> x.lt : (int)blockDim.x;  // 2^lt divides the thread count
   for (int c0 = 0; c0 < (COLS ? 1 : x.lines); ++c0) {
@@ -307,14 +310,16 @@ __device__ __forceinline__ void copy_out(const Ctx<T, COLS, BS>& x, const typena
 // differences s_r = v_r + v_{R-r}, d_r = v_r - v_{R-r} (twiddled) replace
 // them in shared memory; then every thread forms kPairGroup output pairs
 // y_q, y_{R-q} = a -+ i b of one butterfly (see dft_odd; q = 0 is y_0).
-template <typename T, bool COLS, bool BS>
-__device__ void pass_prime(const Ctx<T, COLS, BS>& x, const MixStage& st, int s, bool last,
+template <typename T, bool COLS, bool BS, bool TIGHT>
+__device__ void pass_prime(const Ctx<T, COLS, BS, TIGHT>& x, const MixStage& st, int s, bool last,
                            typename cpx<T>::type* root) {
   using C = typename cpx<T>::type;
   const int R = st.r, H = (R - 1) / 2, nb = st.nb;
   C* src = x.buf(s + 1);
   C* dst = x.buf(s);
-  for (int e = threadIdx.x; e < R; e += blockDim.x) root[e] = x.tw[sizeof(T) == 4 ? st.roff + e : e * (x.len / R)];  // e^{-2 pi i e / R}
+  const auto root_in = [&](int e) -> int { return sizeof(T) == 4 ? st.roff + e : e * (x.len / R); };  // e^{-2 pi i e / R} in tw
+  if (!TIGHT)
+    for (int e = threadIdx.x; e < R; e += blockDim.x) root[e] = x.tw[root_in(e)];
   const int per = x.items(nb);  // items of one value of r
   for (int b = threadIdx.x; b < per * (H + 1); b += blockDim.x) {
     const int r = b / per;
@@ -368,7 +373,7 @@ __device__ void pass_prime(const Ctx<T, COLS, BS>& x, const MixStage& st, int s,
       for (int g = 0; g < kPairGroup; ++g) {
         e[g] += q[g];
         if (e[g] >= R) e[g] -= R;
-        const C w = root[e[g]];  // (cos, -sin); pairs past H read in range and are not stored
+        const C w = TIGHT ? __ldg(&x.tw[root_in(e[g])]) : root[e[g]];  // (cos, -sin); pairs past H read in range and are not stored
         a[g].x = fma(w.x, sv.x, a[g].x);
         a[g].y = fma(w.x, sv.y, a[g].y);
         bb[g].x = fma(w.y, dv.x, bb[g].x);
@@ -412,7 +417,7 @@ constexpr int mix_min_ctas() {
 
 // ROWS: CTA = L consecutive lines.  COLS: CTA = 2^lt neighbouring columns of
 // one slab of [outer][len][inner].
-template <typename T, bool COLS, bool BS>
+template <typename T, bool COLS, bool BS, bool TIGHT>
 __global__ void __launch_bounds__(kMixThreads, mix_min_ctas<T>())
     k_dft_mix(const void* in, int kind, void* out, int out_mode, int64_t nlines, int inner, int L, int lt, int len, MixArgs a,
               int inverse, T scale, double accum_scale, const typename cpx<T>::type* __restrict__ sc_in,
@@ -420,8 +425,12 @@ __global__ void __launch_bounds__(kMixThreads, mix_min_ctas<T>())
   using C = typename cpx<T>::type;
   if (skip && *skip) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ C root[64];
-  Ctx<T, COLS, BS> x;
+  C* root = nullptr;
+  if constexpr (!TIGHT && !BS) {
+    __shared__ C roots[kMixRoots];
+    root = roots;
+  }
+  Ctx<T, COLS, BS, TIGHT> x;
   x.in = in;
   x.out = out;
   x.kind = kind;
@@ -429,7 +438,7 @@ __global__ void __launch_bounds__(kMixThreads, mix_min_ctas<T>())
   x.len = len;
   x.lt = lt;
   x.inner = inner;
-  x.pitch = a.m.n + (a.m.n >> x.kPad) + 1;
+  x.pitch = x.pitch_of(a.m.n);
   if (COLS) {
     const int tiles = (inner + (1 << lt) - 1) >> lt;
     const int slab = blockIdx.x / tiles, c0 = (blockIdx.x - slab * tiles) << lt;
@@ -483,20 +492,28 @@ cudaError_t run_mix(const MixArgs& a, int len, const void* in, int kind, void* o
                     const void* sc_out, const int* skip, cudaStream_t st) {
   using C = typename cpx<T>::type;
   const MixShape h = mix_shape(a.m, COLS, sizeof(C), nlines, outer, inner);
-  const int pad = Ctx<T, COLS, BS>::kPad;
-  const size_t buf = COLS ? ((size_t)a.m.n << h.lt) : (size_t)(a.m.n + (a.m.n >> pad) + 1) * h.L;
-  const size_t smem = buf * h.nbuf * sizeof(C);
   const int64_t grid = COLS ? outer * ((inner + (int64_t(1) << h.lt) - 1) >> h.lt) : (nlines + h.L - 1) / h.L;
   if (grid == 0) return cudaSuccess;
-  auto k = k_dft_mix<T, COLS, BS>;
-  if (smem > 40 * 1024) {
-    const cudaError_t e = allow_dynamic_smem((const void*)k, smem);
-    if (e != cudaSuccess) return e;
-  }
-  k<<<(unsigned)grid, h.threads, smem, st>>>(in, kind, out, out_mode, nlines, (int)inner, h.L, h.lt, len, a,
-                                             sign > 0 ? 1 : 0, (T)scale, accum_scale, (const C*)sc_in,
-                                             (const C*)sc_out, skip);
-  return cudaGetLastError();
+  auto go = [&](auto kern, size_t line) -> cudaError_t {
+    const size_t smem = line * h.L * h.nbuf * sizeof(C);
+    if (smem > 40 * 1024) {
+      const cudaError_t e = allow_dynamic_smem((const void*)kern, smem);
+      if (e != cudaSuccess) return e;
+    }
+    kern<<<(unsigned)grid, h.threads, smem, st>>>(in, kind, out, out_mode, nlines, (int)inner, h.L, h.lt, len, a,
+                                                  sign > 0 ? 1 : 0, (T)scale, accum_scale, (const C*)sc_in,
+                                                  (const C*)sc_out, skip);
+    return cudaGetLastError();
+  };
+  if (COLS) return go(k_dft_mix<T, COLS, BS, false>, a.m.n);  // L = 2^lt columns
+  const size_t padded = Ctx<T, COLS, BS, false>::pitch_of(a.m.n);
+  // The longest rows (6428 .. 7264 points in complex128, 13643 .. 14528 in
+  // complex64, one line a CTA) leave no room for padding or roots: these are
+  // read from global memory.
+  if constexpr (!COLS && !BS)
+    if ((padded * h.L * h.nbuf + kMixRoots) * sizeof(C) > kMixSmem)
+      return go(k_dft_mix<T, COLS, BS, true>, Ctx<T, COLS, BS, true>::pitch_of(a.m.n));
+  return go(k_dft_mix<T, COLS, BS, false>, padded);
 }
 
 }  // namespace helm

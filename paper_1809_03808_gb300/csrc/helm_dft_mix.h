@@ -16,6 +16,11 @@ struct MixArgs {
   const void* bf;  // its spectrum
 };
 
+// Shared memory a CTA can have; dft_supported accepts lengths of which it holds
+// two bare lines.
+constexpr size_t kMixSmem = 227 * 1024;
+constexpr int kMixRoots = 64;  // a prime pass's roots beside the lines
+
 // Lines per CTA, column slots, threads and exchange buffers of one launch.
 struct MixShape {
   int L, lt, threads, nbuf;
