@@ -153,35 +153,34 @@ __device__ __forceinline__ cll dot_cplx(cll s, const cll (&P)[NK], const LimbC* 
   return {fold(fold(s.x, ax), bx), fold(fold(s.y, ay), by)};
 }
 
-// v = h 2^32 + l with l signed (h = 0 whenever v fits l): two 32-bit
-// conversions (one of 64 bits would run on the FP64 pipe).
+// v / 2^32 for v = h 2^32 + l with l signed (h = 0 whenever v fits l): two
+// 32-bit conversions (one of 64 bits would run on the FP64 pipe).
 __device__ __forceinline__ float fx_to_float(ll v) {
   const int l = (int)v, h = (int)(v >> 32) + (int)((uint32_t)l >> 31);
-  return fmaf((float)h, 4294967296.0f, (float)l);
+  return fmaf((float)l, 0x1p-32f, (float)h);
 }
 
-// Factors of the result's unit 2^(K - 1080) (two: K may leave a float's
-// exponents), NaN from a bad key on.
+// Factors of 2^32 units of the result, 2^(K - 1048) (two: K may leave a
+// float's exponents), NaN from a bad key on.
 struct Unit {
   float a, b;
 };
 __device__ __forceinline__ Unit unit_of(int K) {
   if (K >= kBadKey / 2) return {__int_as_float(0x7fffffff), 1.0f};
-  const int s = K - 1080;
+  const int s = K - 1048;
   const int s1 = max(-126, min(127, s)), s2 = max(-126, min(127, s - s1));
   return {__int_as_float((s1 + 127) << 23), __int_as_float((s2 + 127) << 23)};
 }
 
 // What a thread carries along its column: -R(x-1), f - Q - R(x-2) at x-1, and
-// the sums of |r|^2 (in units) and |f|^2 (in 2^32 units, from the high words:
-// 26 bits of the tile's largest value; the norms only decide convergence).
+// the sums of |r|^2 (in 2^32 units: 64 x 32 of them stay in a float's range)
+// and |f|^2.  The latter is of f itself, which may lie far below the tile's
+// terms of A u, and in FP64: two instructions on a pipe that is idle here.
 struct Column {
   cll A = {0, 0}, R = {0, 0};
-  float r2 = 0.f, f2 = 0.f;
-  __device__ __forceinline__ void add_f(cll f) {
-    const float x = (float)(int)(f.x >> 32), y = (float)(int)(f.y >> 32);
-    f2 = fmaf(x, x, fmaf(y, y, f2));
-  }
+  float r2 = 0.f;
+  double f2 = 0.0;
+  __device__ __forceinline__ void add_f(double2 f) { f2 = fma(f.x, f.x, fma(f.y, f.y, f2)); }
   // r at x-1 from -R(x)
   __device__ __forceinline__ float2 finish(cll Rn, Unit un) {
     const float x = fx_to_float(A.x + Rn.x), y = fx_to_float(A.y + Rn.y);
@@ -190,12 +189,11 @@ struct Column {
   }
   // a unit 2^d times larger
   __device__ __forceinline__ void grow(int d) {
+    const float g = __int_as_float((127 - min(d, 126)) << 23);
+    r2 = r2 * g * g;
     d = min(d, 63);
     A = {A.x >> d, A.y >> d};
     R = {R.x >> d, R.y >> d};
-    const float g = __int_as_float((127 - d) << 23);
-    r2 = r2 * g * g;
-    f2 = f2 * g * g;
   }
 };
 
@@ -203,16 +201,16 @@ struct Column {
 template <int NT>
 __device__ __forceinline__ void fx_norms(const Column& c, int K, double* sums, int64_t bid) {
   __shared__ double sr[NT / 32], sf[NT / 32];
-  float r2 = c.r2, f2 = c.f2;
+  float r2 = c.r2;
+  double f2 = c.f2;
   for (int off = 16; off > 0; off >>= 1) {
     r2 += __shfl_down_sync(0xffffffffu, r2, off);
     f2 += __shfl_down_sync(0xffffffffu, f2, off);
   }
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
   if ((tid & 31) == 0) {
-    const bool bad = K >= kBadKey / 2;
-    sr[tid >> 5] = bad ? (double)__int_as_float(0x7fffffff) : scalbn((double)r2, 2 * (K - 1080));
-    sf[tid >> 5] = bad ? (double)__int_as_float(0x7fffffff) : scalbn((double)f2, 2 * (K - 1048));
+    sr[tid >> 5] = K >= kBadKey / 2 ? (double)__int_as_float(0x7fffffff) : scalbn((double)r2, 2 * (K - 1048));
+    sf[tid >> 5] = f2;
   }
   __syncthreads();
   if (tid == 0) {
@@ -349,7 +347,7 @@ __global__ void __launch_bounds__(FT, 2)
     P[3] = (U[0] + U[2]) + (U[2 * FW] + U[2 * FW + 2]);
     const double2 fv = reinterpret_cast<const double2*>(sF + (i % FNB) * FFB)[tid];
     cll A = {to_fx<5>(fv.x, K), to_fx<5>(fv.y, K)}, Rn;  // f - Q, -R
-    if (outp) col.add_f(A);  // zeros outside the grid
+    if (outp) col.add_f(fv);  // zeros outside the grid
     const bool cx = ip == 0 || ip == a.nx - 1;
     if (!face && !cx) {
       dot_real<4>(P, a.q, a.r, A, Rn);
@@ -440,7 +438,7 @@ __global__ void __launch_bounds__(32 * kFx2Warps, 3)
       P[1].x = __shfl_up_sync(0xffffffffu, P[0].x, 1) + __shfl_down_sync(0xffffffffu, P[0].x, 1);
       P[1].y = __shfl_up_sync(0xffffffffu, P[0].y, 1) + __shfl_down_sync(0xffffffffu, P[0].y, 1);
       cll A = {to_fx<5>(fv.x, K), to_fx<5>(fv.y, K)}, Rn;  // f - Q, -R
-      col.add_f(A);  // zero where the lane has no output here
+      col.add_f(fv);  // zero where the lane has no output here
       const bool cx = ip == 0 || ip == a.nx - 1;
       if (!face && !cx) {
         dot_real<2>(P, a.q, a.r, A, Rn);
