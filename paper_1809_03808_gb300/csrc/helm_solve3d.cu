@@ -46,7 +46,7 @@ struct Plane3DArgs {
 
 constexpr int XC = 32;  // rows per reduction chunk
 
-constexpr int kLineVals = 6;  // per-line table values (see k_plane_tables)
+constexpr int kLineVals = 5;  // per-line table values (see k_plane_tables)
 constexpr int kRoutedFlag = 1 << 30;  // in the settling-row table: the line is solved in FP64
 // Routing is off by default: the complex64 solve's error does sit in the
 // near-singular lines (92 % of it in 1 % of the lines on a 160^3 grid of the
@@ -511,10 +511,9 @@ __global__ void k_outer_cbb(const typename cpx<T>::type* __restrict__ v, const t
 // for complex64 tables, a quarter of the FP32 rounding; 2^-50 for
 // complex128), so the tiled sweeps read the table only for rows < len and use
 // 1/u_inf beyond.  Per line (kLineVals values, line = l * nz + m): 1/u_inf,
-// 1/u_{nx-1} (the corner row), the off-diagonal b of the line matrix, and
-// the carry coefficients alpha, beta of a chunk of ch settled rows and beta of
-// the line's last chunk (see k_inner3d), all from the FP64 values.  For
-// propagating modes the pivots keep oscillating and len covers the whole line.
+// the off-diagonal b of the line matrix, and the carry coefficients alpha, beta
+// of a chunk of ch settled rows and beta of the line's last chunk (see
+// k_inner3d), all from the FP64 values.  For propagating modes the pivots keep oscillating and len covers the whole line.
 
 template <typename T>
 __global__ void k_plane_tables(typename cpx<T>::type* __restrict__ tab, typename cpx<T>::type* __restrict__ lend,
@@ -567,11 +566,10 @@ __global__ void k_plane_tables(typename cpx<T>::type* __restrict__ tab, typename
       al = an;
     }
     lend[kLineVals * i] = cvt<C>(iinf);
-    lend[kLineVals * i + 1] = cvt<C>(inv);
-    lend[kLineVals * i + 2] = cvt<C>(k.b);
-    lend[kLineVals * i + 3] = cvt<C>(al);
-    lend[kLineVals * i + 4] = cvt<C>(be);
-    lend[kLineVals * i + 5] = cvt<C>(bel);
+    lend[kLineVals * i + 1] = cvt<C>(k.b);
+    lend[kLineVals * i + 2] = cvt<C>(al);
+    lend[kLineVals * i + 3] = cvt<C>(be);
+    lend[kLineVals * i + 4] = cvt<C>(bel);
     lenL[i] = (int)(last_bad + 1);
   }
 }
@@ -876,11 +874,11 @@ __global__ void __launch_bounds__(MAXT, MINB) k_inner3d(
       }
       // line constants from the plan tables
       const int64_t line = l * nz + mc;
-      lc[t] = lend[kLineVals * line + 2];
+      lc[t] = lend[kLineVals * line + 1];
       lc[kMW + t] = lend[kLineVals * line];
-      lc[2 * kMW + t] = lend[kLineVals * line + 3];
-      lc[3 * kMW + t] = lend[kLineVals * line + 4];
-      lc[4 * kMW + t] = lend[kLineVals * line + 5];
+      lc[2 * kMW + t] = lend[kLineVals * line + 2];
+      lc[3 * kMW + t] = lend[kLineVals * line + 3];
+      lc[4 * kMW + t] = lend[kLineVals * line + 4];
       // a line routed to FP64 (flag bit) gets a zero right-hand side here, so
       // it adds nothing to the faces; the FP64 kernel solves it
       const int lr = on ? lenL[line] : 0;

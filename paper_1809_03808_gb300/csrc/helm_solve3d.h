@@ -27,8 +27,9 @@ struct Plan3D {
   void* partial = nullptr;
   // reciprocal pivots of the inner lines, [outer A][inner A] (nullptr: none)
   void* tab[4] = {nullptr, nullptr, nullptr, nullptr};
-  // per inner line of each type: six values (1/u_inf, 1/u_{nx-1}, b and the
-  // settled chunks' carry coefficients, see k_plane_tables), and the row from which the pivots have settled at 1/u_inf
+  // per inner line of each type: five values (1/u_inf, b and the settled
+  // chunks' carry coefficients, see k_plane_tables), and the row from which the
+  // pivots have settled at 1/u_inf
   void* lend[4] = {nullptr, nullptr, nullptr, nullptr};
   int* lenL[4] = {nullptr, nullptr, nullptr, nullptr};
   // tiled inner sweeps: face partials [ny][nparts][2][nx], inner faces
