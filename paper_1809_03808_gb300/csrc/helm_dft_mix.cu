@@ -102,12 +102,12 @@ MixShape mix_shape(const MixPlan& m, bool cols, size_t es, int64_t nlines, int64
     while (tc > 4 && tc * line > 48 * 1024) tc /= 2;
     while (tc > 1 && tc * line > 160 * 1024) tc /= 2;
     while (tc > 1 && tc / 2 >= inner) tc /= 2;
-    while (tc > 2 && outer * ((inner + tc - 1) / tc) < 2 * 152) tc /= 2;
+    while (tc > 2 && outer * ((inner + tc - 1) / tc) < 2 * kSMs) tc /= 2;
     while ((1 << h.lt) < tc) ++h.lt;
     h.L = tc;
   } else {
     int64_t l = std::min<int64_t>(4096 / m.n, (int64_t)(48 * 1024 / line));
-    l = std::min<int64_t>(l, nlines / (2 * 152));
+    l = std::min<int64_t>(l, nlines / (2 * kSMs));
     h.L = (int)std::max<int64_t>(1, l);
   }
   // threads: the fewest thread slots over all passes (idle slots of the last

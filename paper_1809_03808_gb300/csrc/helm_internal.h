@@ -13,6 +13,7 @@
 namespace helm {
 
 constexpr int kMaxStages = 24;
+constexpr int kSMs = 152;  // SMs of a GB300, in the rules that size launches
 
 // Counted device allocations of plan memory (helm_alloc.cpp): the library
 // allocates and frees device memory only through these.

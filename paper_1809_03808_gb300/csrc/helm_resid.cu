@@ -837,7 +837,7 @@ cudaError_t launch_residual_ff(int dim, const int64_t* n, const double* h, doubl
 
 // One resident wave of 256-thread blocks (8 per SM), fewer for small N.
 static int64_t ew_grid(int64_t N) {
-  int dev = 0, nsm = 152;
+  int dev = 0, nsm = kSMs;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   return std::max<int64_t>(1, std::min<int64_t>((N + 255) / 256, (int64_t)nsm * 8));
 }
@@ -873,7 +873,7 @@ __global__ void k_trial_rhs(double2* __restrict__ f, int64_t N, uint64_t seed) {
 
 cudaError_t launch_trial_rhs(double2* f, int64_t N, uint64_t seed, cudaStream_t st) {
   if (N == 0) return cudaSuccess;
-  const int64_t grid = std::min<int64_t>((N + 255) / 256, 152 * 16);
+  const int64_t grid = std::min<int64_t>((N + 255) / 256, kSMs * 16);
   k_trial_rhs<<<(unsigned)grid, 256, 0, st>>>(f, N, seed);
   return cudaGetLastError();
 }

@@ -462,7 +462,7 @@ __global__ void __launch_bounds__(32 * kFx2Warps, 3)
 int fx2_rows(const int64_t* n) {
   const int64_t cols = (n[1] + kFx2Cols - 1) / kFx2Cols;
   int rows = 64;
-  while (rows > 2 && cols * ((n[0] + rows - 1) / rows) < 152 * 16) rows /= 2;
+  while (rows > 2 && cols * ((n[0] + rows - 1) / rows) < kSMs * 16) rows /= 2;
   return rows;
 }
 

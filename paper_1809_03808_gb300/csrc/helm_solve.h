@@ -61,7 +61,7 @@ cudaError_t launch_tri2d_tab(int step, const void* fhat, const void* faces, cons
 // pass 2 takes 17 us with 128 lines and 14 with 32 (launch and timing 5 of it).
 // Beyond that 128 lines write a quarter of the partials.
 inline int tri2d_tab_lines(int64_t n1, int64_t nchunks) {
-  return (n1 + 127) / 128 * nchunks < 8 * 152 ? 32 : 128;
+  return (n1 + 127) / 128 * nchunks < 8 * kSMs ? 32 : 128;
 }
 // complex64 path with a per-plan pivot table (1/u_j rounded from FP64, chunk
 // constants): table memory per line type, building it, and the step launch.

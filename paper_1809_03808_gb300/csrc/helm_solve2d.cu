@@ -1670,7 +1670,7 @@ int tri2d_fused_lines(int prec, int64_t nx, int64_t n1, int64_t nchunks) {
   if ((size_t)(nx * n1) * (prec == kPrecF64 ? sizeof(double2) : sizeof(float2)) > kFusedBytes) return 0;
   const int lmin = prec == kPrecF64 ? 2 : 4;  // 32 bytes of a row
   // twice that once the blocks of the smaller choice are several per SM
-  const int64_t L = (n1 + 2 * lmin - 1) / (2 * lmin) >= 152 ? 2 * lmin : lmin;
+  const int64_t L = (n1 + 2 * lmin - 1) / (2 * lmin) >= kSMs ? 2 * lmin : lmin;
   for (int64_t t = L; t >= lmin; t /= 2)
     if (t * nchunks <= kFusedThreads) return (int)t;
   return 0;

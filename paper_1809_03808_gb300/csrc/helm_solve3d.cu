@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(1024) k_plane3d(const typename cpx<T>::type* _
 // FP64 pipe in complex128 (201 x 150 x 175: 94 us, now 88).
 constexpr int kOuterChunk = 1024;
 constexpr int kOuterBatch = 8;
-constexpr int64_t kOuterSplitBelow = 152 * 1024;
+constexpr int64_t kOuterSplitBelow = kSMs * 1024;
 template <typename T, int OSTEP, int SPLIT>
 __global__ void __launch_bounds__(256) k_reduce_outer(const typename cpx<T>::type* __restrict__ y3,
                                                       typename cpx<T>::type* __restrict__ out, Plane3DArgs a,
@@ -1678,7 +1678,7 @@ cudaError_t plan3d_init(Plan3D& p, int prec, const int64_t* n, const double* h, 
     // tiles per CTA: one, and two where that still leaves 32 CTAs for an SM
     // (512^3: half the face partials to reduce; 384 x 320 x 256 is 4 % faster
     // with one)
-    int nmb = prec == kPrecF32 && total >= 2 * 152 * 32 ? 2 : 1;
+    int nmb = prec == kPrecF32 && total >= 2 * kSMs * 32 ? 2 : 1;
     nmb = (int)std::min<int64_t>(nmb, tiles);
     const int nparts = (int)((tiles + nmb - 1) / nmb);
     const size_t sz[3] = {(size_t)n[1] * nparts * 2 * n[0] * cb, (size_t)n[1] * 4 * n[0] * cb,
