@@ -721,14 +721,15 @@ cudaError_t launch_residual(int dim, const int64_t* n, const double* h, double o
                   if (a1 == 0) put(q.c0[4 * cx + 2 * cy + cz][2 * b + c], v);
                   else if (cx == 0) put(q.c1[2 * cy + cz][2 * b + c], v);
                 }
+      const cudaError_t e = launch_residual_fx(3, q, f, u, r, sums, nblocks, skip, err, st);
+      if (e != cudaErrorNotSupported) return e;
+      // no tensor maps: the FP64 kernel, with its class corrections
       for (int cls = 0; cls < 8; ++cls)
         for (int bc = 0; bc < 4; ++bc) {
           q.dc0[cls][bc] = make_double2(q.c0[cls][bc].x - q.c0[cls & 4][bc].x, q.c0[cls][bc].y - q.c0[cls & 4][bc].y);
           if (cls < 4)
             q.dc1[cls][bc] = make_double2(q.c1[cls][bc].x - q.c1[0][bc].x, q.c1[cls][bc].y - q.c1[0][bc].y);
         }
-      const cudaError_t e = launch_residual_fx(3, q, f, u, r, sums, nblocks, skip, err, st);
-      if (e != cudaErrorNotSupported) return e;
       const dim3 grid((unsigned)((n[2] + QZ - 1) / QZ), (unsigned)((n[1] + QY - 1) / QY), (unsigned)((n[0] + QX - 1) / QX));
       *nblocks = (int64_t)grid.x * grid.y * grid.z;
       k_residual3d_q<<<grid, dim3(QZ, QY), 0, st>>>(q, f, u, r, sums, skip);
