@@ -153,12 +153,30 @@ class ClockSampler:
 # writes, e = bytes per complex value of the compute precision (16 FP64, 8
 # FP32); the first solve reads f as complex128, refinement sweeps read the
 # complex64 residual, the last transform writes (or updates) complex128 u.
-# Flops: real operations of the algorithm as written (complex multiply 6,
-# complex add 2, complex reciprocal 5 counting each division as 1).
+# Flops: complex64 kernels, real operations of the algorithm as written
+# (complex multiply 6, complex add 2, complex reciprocal 5 counting each
+# division as 1); complex128 kernels, FP64 instructions as their code forms
+# them, a fused multiply-add counting once as in the peak they are held
+# against (complex multiply or multiply-add 4, add or scaling 2).
+def fp64_dft_ops(n):
+    """FP64 instructions per point of a transform of n = 2^m points: one pass
+    of radix 2 .. 16, then radix-16 passes with their twiddles (15 complex
+    multiplies per 16 points), and the scalings (one real, one complex)."""
+    import math
+
+    m = round(math.log2(n))
+    if 1 << m != n:
+        return 5.0 * math.log2(n)
+    first = {1: 2.0, 2: 4.0, 3: 7.0, 4: 10.0}[(m - 1) % 4 + 1]
+    return first + (m - 1) // 4 * (3.75 + 10.0) + 6.0
+
+
 def kernel_model(name, e, n1, accum=False, first=True, tables=False, ff=False, per_solve=1.0, n1_dim=2):
     import math
 
     log2n = math.log2(n1)
+    c128 = e == 16
+    dft = fp64_dft_ops(n1) if c128 else 5.0 * log2n
     # forward-transform input, averaged over the per_solve launches of a
     # refined solve: the first reads f (complex128; with the float-float
     # residual the complex64 hi parts the split wrote), the sweeps read r
@@ -166,10 +184,12 @@ def kernel_model(name, e, n1, accum=False, first=True, tables=False, ff=False, p
     fin = (f0 + (per_solve - 1.0) * e) / per_solve if first else e
     if tables:
         # FP64 with per-plan line tables: pass 1 reads rhs, m_j, w_j; pass 2
-        # reads rhs, m_j, 1/u_j (and step 3 writes x)
-        tri = {"tri_step1_pass1": (3 * e, 22.0), "tri_step2_pass1": (2 * e, 18.0),
-               "tri_step3_pass1": (3 * e, 24.0), "tri_step1_pass2": (3 * e, 34.0),
-               "tri_step2_pass2": (2 * e, 36.0), "tri_step3_pass2": (4 * e, 30.0)}
+        # reads rhs, m_j, 1/u_j (and step 3 writes x).  Instructions: the rhs
+        # (4, 2, 12), then 7.5 in pass 1 (a chunk's first row has no carry) and 12
+        # in pass 2, with 8 for the faces (Step 2: 10)
+        tri = {"tri_step1_pass1": (3 * e, 11.5), "tri_step2_pass1": (2 * e, 9.5),
+               "tri_step3_pass1": (3 * e, 19.5), "tri_step1_pass2": (3 * e, 24.0),
+               "tri_step2_pass2": (2 * e, 24.0), "tri_step3_pass2": (4 * e, 24.0)}
     else:
         # complex64: the rhs (f_hat; Step 2 only face vectors) and, in Step 3,
         # the solution; the per-plan 1/u_j table is read only for rows before
@@ -180,34 +200,36 @@ def kernel_model(name, e, n1, accum=False, first=True, tables=False, ff=False, p
     # on columns; k_plane3d per outer step: per inner step the forward sweep
     # reads 1/den and writes d, the backward sweep reads both (4e), x3 steps,
     # plus f_hat read in inner Steps 1 and 3 (outer Steps 1, 3) and y3 written
-    c128 = e == 16
     # tiled inner sweeps (3D): the rhs read from f_hat in outer Steps 1, 3
     # (inner Steps 1, 3), y3 written in inner Step 3; inner Step 2 and outer
     # Step 2 generate their right-hand sides from face vectors (no bulk bytes)
     if name.startswith("inner_o") and len(name) == 11:
         o, i = int(name[7]), int(name[10])
         byts = (e if (o != 2 and i != 2) else 0.0) + (e if i == 3 else 0.0)
-        return (byts, 80.0) if byts > 0 else None
+        # complex128: the rhs (outer faces 2 to 6, C_bb terms 8), 4 each for the
+        # two sweeps of pass 1, 10 for pass 2, 6 for the faces of inner Step 1
+        ops = {1: 4.0, 2: 6.0, 3: 10.0}[o] + 18.0 + (8.0 if i != 1 else 0.0) + (6.0 if i == 1 else 0.0)
+        return (byts, ops if c128 else 80.0) if byts > 0 else None
     tab3 = {
-        "dft_z_fwd": ((16 if c128 else 8) + e, 5.0 * log2n),
-        "dft_y_fwd": (2 * e, 5.0 * log2n),
-        "dft_y_inv": (2 * e, 5.0 * log2n),
-        "dft_z_inv": (e + (16 if c128 else 32), 5.0 * log2n),
+        "dft_z_fwd": ((16 if c128 else 8) + e, dft),
+        "dft_y_fwd": (2 * e, dft),
+        "dft_y_inv": (2 * e, dft),
+        "dft_z_inv": (e + (16 if c128 else 32), dft),
         "plane3d_step1": (15 * e, 100.0),
         "plane3d_step2": (13 * e, 90.0),
         "plane3d_step3": (15 * e, 100.0),
-        "reduce_outer": (e, 8.0),
+        "reduce_outer": (e, 6.0 if c128 else 8.0),
     }
     if name in tab3:
         return tab3[name]
     tab = {
-        "dft_fwd": (fin + e, 5.0 * log2n),
+        "dft_fwd": (fin + e, dft),
         # refined paths: the first solve writes u (16 B), the sweeps update it (32 B)
         "dft_inv": (e + ((16.0 + (per_solve - 1.0) * 32.0) / per_solve if accum else 16 if e == 16 else 8),
-                    5.0 * log2n),
+                    dft),
         # f, u complex128 in, r complex64 out; 64-bit fixed point on the integer
-        # pipes: no FP64 instructions in its loop
-        "residual_fp64": (40.0, 0.0),
+        # pipes, but for |f|^2: two FP64 instructions
+        "residual_fp64": (40.0, 2.0),
         # f, u float-float (16 B each) in, r complex64 out
         "residual_ff": (40.0, 40.0),
         "split_ff": (40.0, 4.0),  # f in, float-float f and its hi parts out
@@ -229,7 +251,7 @@ NCU_TRAFFIC_PER_UNKNOWN = {
     # DRAM bytes of one k_residual3d_fx launch on 128 x 512 x 512, per unknown;
     # the traffic of a launch is proportional to them
     ("3d", "c64_refined", "residual_fp64"): (
-        (1107.046656e6 + 252.338432e6) / (128 * 512 * 512),
+        (1106.899456e6 + 256.080128e6) / (128 * 512 * 512),
         "ncu, 128 x 512 x 512: k_residual3d_fx (profiles/ncu_residual3d_fx.md), scaled by unknowns"),
 }
 

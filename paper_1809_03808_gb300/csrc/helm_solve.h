@@ -99,10 +99,10 @@ struct RefineState {
   double resid[16];
 };
 
-// r = f - A u of FP64 vectors (eq. A2D / A3D) in 64-bit fixed point, at least
-// FP64's accuracy (helm_resid_fx.cu), r stored as complex64, per-block sums
-// of |r|^2 and |f|^2 into `sums` (2 doubles per block).  Returns the number of
-// blocks used through *nblocks.
+// r = f - A u of FP64 vectors (eq. A2D / A3D) in 64-bit fixed point, with errors
+// of about 2^-58 of the largest sum |c| |u| of a tile (helm_resid_fx.cu), r
+// stored as complex64, per-block sums of |r|^2 and |f|^2 into `sums` (2 doubles
+// per block).  Returns the number of blocks used through *nblocks.
 // wc[k]: w of the absorbing ends of axis k (0 on a Neumann axis).  err: the
 // device error word set if a bounded wait of the 3D kernel runs out.  mden:
 // the mass matrix denominator of the elements (MassCoef).
